@@ -83,6 +83,12 @@ typedef enum {
  *               fp16 range (65504) is detected: finalize / tacaw_check_errors then return
  *               TACAW_ERR_OVERFLOW and the plan is poisoned.  Staged operands only
  *               (frames_in_place must be 0).
+ * Band-limited staging (staged plans with 32-frame blocks, or FP32; segments of 512 frames and more):
+ * where the energies cover less than half of the band 1/dt, pushes may stage blocks of 32, 64 or 128
+ * frames as their fewer coefficients on an orthonormal basis of that band (reconstruction error
+ * 1e-7), which the contraction sums like frames.  The first push into a staging ring picks the form by
+ * its length.  On both split paths the coefficients are fp16 hi + lo pieces under a power-of-two scale
+ * per row, whatever the pieces of staged frames are; no input is refused for it.
  * Twiddle phases are always reduced in FP64; the exact mean correction is FP64-derived. */
 typedef enum { TACAW_PREC_FP32 = 0, TACAW_PREC_SPLIT_BF16 = 1, TACAW_PREC_SPLIT_FP16 = 2 } tacaw_precision;
 
@@ -364,7 +370,8 @@ tacaw_status tacaw_reset(tacaw_plan_t plan, void *stream);
  *   so far): a 48-byte header, 48 bytes per internal stream (Welch lanes count one each) and 8
  *   per stream, then the device sections.  Per internal stream: the provisional mean (8 bytes a
  *   ROI row) and FP64 residual sums (16 a row); the staged frames not yet contracted (whole
- *   blocks of the staging layout: 8 bytes a row and frame); once a flush has written them, the
+ *   blocks of the staging layout: 8 bytes a row and frame, or a coefficient of band-limited
+ *   staging, 4 a row for its scales, and 8 a row and frame of an unfinished block); once a flush has written them, the
  *   Psi accumulators of the Nw energies (8 bytes a row and energy for FP32 accumulators, 16 for
  *   compensated FP32 or FP64).  Per Welch-averaged stream its running average of I (4 bytes an
  *   element).

@@ -217,6 +217,112 @@ __global__ void window_values_kernel(TableArgs a, float *w) {
     if (t < a.T) w[t] = (float)window_value(a, t);
 }
 
+// ---- band-limited staging form ----------------------------------------------------------
+// Psi_j = sum_t y_t w_t exp(-2 pi i c_j t) block by block: with t = t0 + u inside a block of B frames,
+// centre c = (B-1)/2, and m[t] = w_t exp(-2 pi i f_c (u - c)),
+//   sum_u y w exp(-2 pi i c_j t) = exp(-2 pi i c_j (t0 + c)) sum_u (m y)_u exp(-2 pi i (c_j - f_c)(u - c))
+// and the last exponential, |c_j - f_c| <= beta/2, is expanded on the R basis vectors v_q (real,
+// orthonormal, even or odd): its coefficients are q_resp[q][j] = sum_u v_q[u] exp(-2 pi i d (u - c)),
+//   even: 2 sum_{u < B/2} v cos(2 pi d (u - c)),   odd: -2 i sum_{u < B/2} v sin(2 pi d (u - c)).
+
+__global__ void band_mod_kernel(TableArgs a, int B, double fc, int n, float2 *mod) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= n) return;
+    float2 v = make_float2(0.f, 0.f);
+    if (t < a.T) {
+        double c, s;
+        sincospi(2.0 * fc * ((double)(t % B) - 0.5 * (double)(B - 1)), &s, &c);
+        const double w = window_value(a, t);
+        v = make_float2((float)(w * c), (float)(-w * s));
+    }
+    mod[t] = v;
+}
+
+// one thread per (energy, basis vector); a.cj holds c_j for FFT grids too
+__global__ void band_response_kernel(TableArgs a, BandTableArgs b, double *q_resp) {
+    const int j = blockIdx.x * blockDim.x + threadIdx.x, q = blockIdx.y;
+    if (j >= a.Nw) return;
+    const double d = a.cj[j] - b.fc;
+    double acc = 0.0;
+    for (int u = 0; u < b.B / 2; ++u) {
+        double c, s;
+        sincospi(2.0 * d * ((double)u - 0.5 * (double)(b.B - 1)), &s, &c);
+        acc += b.basis[u * b.R + q] * (q >= b.R / 2 ? -2.0 * s : 2.0 * c);
+    }
+    q_resp[(size_t)q * a.Nw + j] = acc;
+}
+
+// One thread per (energy j < Nw_pad, block): the R table rows of block k of flush f.  The split path
+// takes fp16 pieces (|B| is at most about sqrt(B)).
+__global__ void band_twiddles_kernel(TableArgs a, BandTableArgs b, const double *q_resp, __nv_bfloat16 *B_hi,
+                                     __nv_bfloat16 *B_lo, float2 *B32) {
+    const int per = (b.slots + b.R - 1) / b.R;      // blocks a flush's table rows hold (the last may be padding)
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    const int n = blockIdx.y * blockDim.y + threadIdx.y;
+    if (j >= a.Nw_pad || n >= b.rounds * per) return;
+    const int f = n / per, k = n % per;
+    const long long t0 = (long long)f * b.ring + (long long)k * b.B;
+    const bool in = j < a.Nw && k * b.B < b.ring && t0 < a.T;
+    double c = 0.0, s = 0.0;
+    if (in) {
+        // phase at the block's centre, in half frames: c_j (2 t0 + B - 1) / 2
+        const long long h = 2 * t0 + b.B - 1;
+        if (a.fft_bins) {
+            const long long r = ((long long)j * h) % (2LL * a.T);
+            sincospi((double)r / (double)a.T, &s, &c);
+        } else {
+            const double x = a.cj[j] * 0.5 * (double)h;
+            sincospi(2.0 * (x - floor(x)), &s, &c);
+        }
+    }
+    const size_t rows = 2 * (size_t)a.Nw_pad;
+    const int n0 = 2 * j, n1 = 2 * j + 1;
+    for (int q = 0; q < b.R && k * b.R + q < b.slots; ++q) {
+        const double g = in ? q_resp[(size_t)q * a.Nw + j] : 0.0;
+        // (c - i s) g, times i for the odd vectors (whose q_resp is the imaginary part)
+        const bool odd = q >= b.R / 2;
+        const float br = (float)(odd ? s * g : c * g), bi = (float)(odd ? c * g : -s * g);
+        const int row = f * b.slots + k * b.R + q;
+        if (B32) {
+            B32[(size_t)row * a.Nw_pad + j] = make_float2(br, bi);
+            continue;
+        }
+        const int kb = row / 32, tt = row % 32;
+        const int w0 = (((tt >> 2) ^ (n0 & 7)) << 2) | (tt & 3), w1 = (((tt >> 2) ^ (n1 & 7)) << 2) | (tt & 3);
+        const size_t r0 = ((size_t)kb * rows + (size_t)n0) * 64 + 2 * (size_t)w0;
+        const size_t r1 = ((size_t)kb * rows + (size_t)n1) * 64 + 2 * (size_t)w1;
+        const float v0[2] = {br, -bi}, v1[2] = {bi, br};
+        for (int e = 0; e < 2; ++e) {
+            __nv_bfloat16 h, l;
+            split_f16(v0[e], h, l);
+            B_hi[r0 + e] = h;
+            B_lo[r0 + e] = l;
+            split_f16(v1[e], h, l);
+            B_hi[r1 + e] = h;
+            B_lo[r1 + e] = l;
+        }
+    }
+}
+
+cudaError_t launch_band_mod(const TableArgs &t, const BandTableArgs &b, float2 *mod, cudaStream_t st) {
+    const int n = (t.T + b.B - 1) / b.B * b.B;
+    band_mod_kernel<<<(n + 127) / 128, 128, 0, st>>>(t, b.B, b.fc, n, mod);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_band_response(const TableArgs &t, const BandTableArgs &b, double *q_resp, cudaStream_t st) {
+    band_response_kernel<<<dim3((t.Nw + 63) / 64, b.R), 64, 0, st>>>(t, b, q_resp);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_band_twiddles(const TableArgs &t, const BandTableArgs &b, const double *q_resp,
+                                 __nv_bfloat16 *B_hi, __nv_bfloat16 *B_lo, float2 *B32, cudaStream_t st) {
+    const dim3 blk(32, 8);
+    const dim3 grd((t.Nw_pad + 31) / 32, (b.rounds * ((b.slots + b.R - 1) / b.R) + 7) / 8);
+    band_twiddles_kernel<<<grd, blk, 0, st>>>(t, b, q_resp, B_hi, B_lo, B32);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_twiddles_split(const TableArgs &t, __nv_bfloat16 *B_hi, __nv_bfloat16 *B_lo, int f16,
                                   cudaStream_t st) {
     dim3 blk(32, 8);

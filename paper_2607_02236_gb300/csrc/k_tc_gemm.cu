@@ -303,6 +303,12 @@ __device__ __forceinline__ void tc_epilogue_prefetch(const TcPlanArgs &a, int64_
     }
 }
 
+// What a row's sums over band-limited coefficients are multiplied by (powers of two).
+__device__ __forceinline__ float row_factor(const TcPlanArgs &a, int64_t m) {
+    const float s = a.row_scale[m];
+    return a.row_unit / (s == 0.f ? 1.f : s);
+}
+
 // Flush epilogue of the split drained form: the tile's result is all in the running sums.
 template <int KIND, int C>
 __device__ __forceinline__ void tc_epilogue_regs(const TcPlanArgs &a, const RowCtx &row, int col0, int cols,
@@ -424,6 +430,9 @@ __device__ __forceinline__ int group_entry(const TcGroup &g, int64_t tile) {
     return gi;
 }
 
+// BAND: some entry's rows are scaled (band-limited staging); launches without one keep an epilogue
+// without the multiplications (they cost short tiles a hundredth).
+template <bool BAND>
 __global__ void __maxnreg__(168) flush_tc_drain2_kernel(const __grid_constant__ TcGroup g) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -699,6 +708,11 @@ __global__ void __maxnreg__(168) flush_tc_drain2_kernel(const __grid_constant__ 
                     sum[2 * i] = v.x;
                     sum[2 * i + 1] = v.y;
                 }
+                if (BAND && preload && a.row_scale) {
+                    const float ps = 1.f / row_factor(a, mrow);
+#pragma unroll
+                    for (int i = 0; i < kDrainCols; ++i) sum[i] *= ps;
+                }
             }
             for (int lc = 0; lc + 1 < n_chunks; ++lc, ++hc) {
                 if (!mbar_wait(smem_u32(&sh->chunk_full[0]), (uint32_t)(hc & 1), abort_flag, wait_ns)) {
@@ -729,6 +743,11 @@ __global__ void __maxnreg__(168) flush_tc_drain2_kernel(const __grid_constant__ 
             if (lane == 0) mbar_arrive(smem_u32(&sh->chunk_free[1]));
             const RowCtx row = make_row(a.e, (int64_t)m0 + q4 * 32 + lane);
             const int jbase = wtile * a.wt;
+            if (BAND && a.row_scale) {
+                const float rf = row_factor(a, row.m);
+#pragma unroll
+                for (int i = 0; i < kDrainCols; ++i) sum[i] *= rf;
+            }
             // with preloaded sums an update of the accumulators is a store, a finalize one without
             // earlier flushes
             const int kind = preload ? (kind0 == EPI_ADD_KAHAN ? EPI_STORE_KAHAN : EPI_FINAL) : kind0;
@@ -1393,9 +1412,9 @@ cudaError_t launch_flush_tc_inplace(const TcPlanArgs &a, const TcDirectArgs &d, 
 int tc_resident_ctas(int N, int bf, int stages) {
     const size_t smem = tc_smem_bytes(N, bf, stages);
     int n = 0;
-    if (cudaFuncSetAttribute(flush_tc_drain2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
+    if (cudaFuncSetAttribute(flush_tc_drain2_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
             cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, flush_tc_drain2_kernel, 320, smem) != cudaSuccess) {
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, flush_tc_drain2_kernel<false>, 320, smem) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
@@ -1445,13 +1464,16 @@ static cudaError_t launch_flush_tc_group_impl(const TcPlanArgs *args, int n, con
     g->stages = tc_stages_for(n_max, args[0].bf);
     g->tiles = total;
     const size_t smem = tc_smem_bytes(n_max, args[0].bf, g->stages);
+    bool band = false;
+    for (int i = 0; i < n; ++i) band = band || args[i].row_scale;
+    void (*kern)(TcGroup) = band ? flush_tc_drain2_kernel<true> : flush_tc_drain2_kernel<false>;
     int dev = 0, sms = 0, occ = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(flush_tc_drain2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, flush_tc_drain2_kernel, threads, smem);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, threads, smem);
     if (e != cudaSuccess || g->stages < 2 || n_max > 2 * kDrainCols || occ < 1) {
         delete g;
         return e != cudaSuccess ? e : cudaErrorInvalidConfiguration;
@@ -1463,7 +1485,7 @@ static cudaError_t launch_flush_tc_group_impl(const TcPlanArgs *args, int n, con
     g->counter = args[0].tile_counter;
     e = cudaMemsetAsync(g->counter, 0, sizeof(int), st);
     if (e == cudaSuccess && conv) e = cudaMemsetAsync(conv->counter, 0, sizeof(int), st);
-    if (e == cudaSuccess) e = launch_persistent(flush_tc_drain2_kernel, grid, (unsigned)threads, smem, st, *g);
+    if (e == cudaSuccess) e = launch_persistent(kern, grid, (unsigned)threads, smem, st, *g);
     delete g;
     return e;
 }

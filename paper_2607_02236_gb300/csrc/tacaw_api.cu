@@ -228,7 +228,8 @@ EpiArgs epi_args(tacaw_plan_s *p, const Stream &s, int mode, float *I_out, float
 
 // Tensor-core arguments of one flush of the s.staged frames of stream s.
 TcPlanArgs tc_args(tacaw_plan_s *p, const Stream &s, const EpiArgs &e) {
-    const int n = s.staged;
+    const int n = s.ring_slots();
+    const BandForm *band = s.form >= 0 ? &s.band[s.form] : nullptr;
     TcPlanArgs a{};
     a.e = e;
     a.wt = s.wt;
@@ -241,19 +242,23 @@ TcPlanArgs tc_args(tacaw_plan_s *p, const Stream &s, const EpiArgs &e) {
         a.N_last = std::min(a.N, (2 * last + 15) / 16 * 16);
     }
     a.n_kb = (n + p->bf - 1) / p->bf;
-    a.kbB0 = s.stage_start / p->bf;
+    a.kbB0 = band ? s.stage_start / s.ring * (band->slots / p->bf) : s.stage_start / p->bf;
     a.bf = p->bf;
     a.stages = s.stages;
-    a.drain_kb = p->drain_kb;
+    // coefficients sum more coherently than frames: chunks of at most 10 blocks keep the truncation of the
+    // tensor core's sums (the error grows with the chunk: 2.6e-6 at 16 blocks, 1.3e-6 at 8 on the scan)
+    a.drain_kb = band ? std::min(p->drain_kb, kBandDrainBlocks) : p->drain_kb;
     a.A_hi = s.A_hi;
     a.A_lo = s.A_lo;
-    a.B_hi = s.B_hi;
-    a.B_lo = s.B_lo;
+    a.B_hi = band ? band->B_hi : s.B_hi;
+    a.B_lo = band ? band->B_lo : s.B_lo;
     a.a_rows = s.M_pad;
     a.b_rows = 2 * s.Nw_pad;
     a.max_ctas = p->tc_max_ctas;
     a.wait_ns = p->wait_ns;
-    a.f16 = p->f16;
+    a.f16 = band || p->f16;
+    a.row_scale = band ? s.row_scale() : nullptr;
+    a.row_unit = p->f16_scale;
     a.err = p->d_err;
     a.trace = nullptr;
     return a;
@@ -298,6 +303,7 @@ void flush_done(tacaw_plan_s *p, Stream &s) {
     p->flushes_total++;
     s.stage_start += s.staged;
     s.staged = 0;
+    s.form = -1;
 }
 
 // Address of frame `a` when frames [a, a + n) of the segment are evenly spaced (pitch_frame
@@ -362,7 +368,7 @@ tacaw_status run_flush(tacaw_plan_s *p, Stream &s, int mode, float *I_out, float
         p->launches++;
         p->flush_launches++;
     } else if (p->prec == TACAW_PREC_SPLIT_BF16) {
-        if (n % p->bf) {
+        if (s.form < 0 && n % p->bf) {   // (the push that completes a band-limited ring zeroes its tail)
             CU_CHECK(p, launch_zero_tail_split(s.M_pad, n, p->bf, s.A_hi, s.A_lo, 1, st), "zero_tail");
             p->launches++;
         }
@@ -376,11 +382,12 @@ tacaw_status run_flush(tacaw_plan_s *p, Stream &s, int mode, float *I_out, float
     } else {
         SimtArgs a{};
         a.e = e;
+        const BandForm *band = s.form >= 0 ? &s.band[s.form] : nullptr;
         a.A32 = s.A32;
-        a.B32 = s.B32;
+        a.B32 = band ? band->B32 : s.B32;
         a.Nw_pad = s.Nw_pad;
-        a.n_frames = n;
-        a.t0 = s.stage_start;
+        a.n_frames = s.ring_slots();
+        a.t0 = band ? s.stage_start / s.ring * band->slots : s.stage_start;
         CU_CHECK(p, launch_flush_simt(a, st), "flush (fp32)");
         p->launches++;
         p->flush_launches++;
@@ -405,7 +412,7 @@ struct FlushReq {
 tacaw_status flush_grouped(tacaw_plan_s *p, std::vector<FlushReq> req, cudaStream_t st) {
     auto work = [&](const FlushReq &q) {
         const Stream &s = p->s[q.s];
-        return (int64_t)((s.staged + p->bf - 1) / p->bf) * (2 * s.wt + 48);
+        return (int64_t)((s.ring_slots() + p->bf - 1) / p->bf) * (2 * s.wt + 48);
     };
     std::stable_sort(req.begin(), req.end(), [&](const FlushReq &a, const FlushReq &b) { return work(a) > work(b); });
     for (size_t g0 = 0; g0 < req.size(); g0 += kMaxGroupStreams) {
@@ -415,7 +422,7 @@ tacaw_status flush_grouped(tacaw_plan_s *p, std::vector<FlushReq> req, cudaStrea
         int64_t nc = 0;
         for (size_t k = g0; k < g1; ++k) {
             Stream &s = p->s[req[k].s];
-            if (s.staged % p->bf) {
+            if (s.form < 0 && s.staged % p->bf) {
                 CU_CHECK(p, launch_zero_tail_split(s.M_pad, s.staged, p->bf, s.A_hi, s.A_lo, 1, st), "zero_tail");
                 p->launches++;
             }
@@ -815,7 +822,7 @@ tacaw_status launch_pending(tacaw_plan_s *p, const Stream *conv, cudaStream_t st
 tacaw_status finalize_pipelined(tacaw_plan_s *p, float *d_I, float *d_S, float2 *d_Psi, cudaStream_t st) {
     Stream &s = p->s[0];
     if (p->pend.active) {
-        tacaw_status r = launch_pending(p, p->deferred_pushes ? &s : nullptr, st);
+        tacaw_status r = launch_pending(p, p->deferred_pushes && s.form < 0 ? &s : nullptr, st);
         if (r != TACAW_OK) return r;
     }
     p->pend.snap = s;
@@ -918,8 +925,7 @@ tacaw_status finalize_impl(tacaw_plan_t p, float *d_I, float *d_S, void *d_Psi, 
     return TACAW_OK;
 }
 
-// Pushes n frames (device pointer, the stream's layout) into internal stream s.
-tacaw_status push_internal(tacaw_plan_s *p, Stream &s, const float2 *frames, int n_frames, cudaStream_t st) {
+FrameGeom push_geom(const Stream &s, const float2 *frames) {
     FrameGeom g{};
     g.pitch_row = s.d.pitch_row;
     g.pitch_frame = s.d.pitch_frame;
@@ -931,6 +937,56 @@ tacaw_status push_internal(tacaw_plan_s *p, Stream &s, const float2 *frames, int
     g.npix = s.npix;
     g.M = s.M;
     g.base = frames;
+    return g;
+}
+
+// Counts a grouped push whose conversion is enqueued; a ring that filled is flushed as after a single push.
+tacaw_status push_counted(tacaw_plan_s *p, UserStream &u, int n, cudaStream_t st) {
+    Stream &s = p->s[u.first];
+    s.staged += n;
+    s.pushed += n;
+    u.pushed += n;
+    if (s.staged == s.ring && s.pushed < s.T) {
+        if (!deferrable(p, s)) return run_flush(p, s, s.flushes == 0 ? FLUSH_STORE : FLUSH_ADD, nullptr, nullptr, st);
+        s.due = true;
+        s.due_stream = st;
+    }
+    return TACAW_OK;
+}
+
+// The conversion of one push of n frames (inside the ring) on the ring's band-limited form.
+ProjEntry proj_entry(const tacaw_plan_s *p, const Stream &s, const FrameGeom &g, int n) {
+    const BandForm &b = s.band[s.form];
+    const bool last = s.pushed + n == s.T;
+    ProjEntry e{};
+    e.g = g;
+    e.n = n;
+    e.c0 = s.staged % b.B;
+    e.nblk = last ? (e.c0 + n + b.B - 1) / b.B : (e.c0 + n) / b.B;
+    const int blk0 = s.staged / b.B, end = (blk0 + e.nblk) * b.R;
+    e.t_block = s.stage_start + blk0 * b.B;
+    e.slot0 = blk0 * b.R;
+    // the ring's last block zeroes the rest of its 32-slot row (split path)
+    e.zero_slots = s.A32 || (!last && s.staged + n != s.ring) ? 0 : (int)round_up(end, 32) - end;
+    e.M_pad = s.M_pad;
+    e.mu_hat = s.mu_hat;
+    e.sum_res = s.sum_res;
+    e.carry = s.carry();
+    e.mod = b.mod;
+    e.A_hi = s.A_hi;
+    e.A_lo = s.A_lo;
+    e.A32 = s.A32;
+    e.row_scale = s.row_scale();
+    if (p->f16) {
+        e.f16_scale = p->f16_scale;
+        e.err = p->d_err;
+    }
+    return e;
+}
+
+// Pushes n frames (device pointer, the stream's layout) into internal stream s.
+tacaw_status push_internal(tacaw_plan_s *p, Stream &s, const float2 *frames, int n_frames, cudaStream_t st) {
+    const FrameGeom g = push_geom(s, frames);
     if (s.due) {
         // this stream's ring is full: its deferred flush (with any others) goes first
         tacaw_status r = flush_due(p, st);
@@ -940,7 +996,12 @@ tacaw_status push_internal(tacaw_plan_s *p, Stream &s, const float2 *frames, int
         CU_CHECK(p, launch_mean(g, n_frames, s.mu_hat, st), "provisional mean");
         p->launches++;
     }
-    if (p->pipe && p->pend.active) {
+    if (s.staged == 0) s.form = choose_form(p, s, std::min(n_frames, s.ring));
+    if (p->pipe && p->pend.active && s.form >= 0) {
+        // band-limited forms are converted at push time (into the staging area the pending
+        // contraction does not read); the pending contraction still goes out with the finalize
+        p->deferred_pushes = true;
+    } else if (p->pipe && p->pend.active) {
         // pipelined segments: the pending contraction's launch converts this segment's frames;
         // here only their addresses are recorded (by a kernel on the stream)
         CU_CHECK(p, launch_frame_table(s.d_frame_ptr + s.pushed, frames, g.pitch_frame, n_frames, st), "frame table");
@@ -953,6 +1014,7 @@ tacaw_status push_internal(tacaw_plan_s *p, Stream &s, const float2 *frames, int
     int done = 0;
     while (done < n_frames) {
         const int chunk = std::min(n_frames - done, s.ring - s.staged);
+        if (s.staged == 0) s.form = choose_form(p, s, chunk);
         FrameGeom gc = g;
         gc.base = g.base + (int64_t)done * g.pitch_frame;
         if (p->in_place) {
@@ -963,7 +1025,14 @@ tacaw_status push_internal(tacaw_plan_s *p, Stream &s, const float2 *frames, int
             CU_CHECK(p, launch_frame_table(s.d_frame_ptr + s.pushed, gc.base, g.pitch_frame, chunk, st), "frame table");
             p->launches++;
         } else {
-            if (p->prec == TACAW_PREC_SPLIT_BF16)
+            if (s.form >= 0) {
+                ProjGroup pg;
+                pg.n = 1;
+                pg.e[0] = proj_entry(p, s, gc, chunk);
+                const BandForm &b = s.band[s.form];
+                std::copy(b.basis.begin(), b.basis.end(), pg.basis);
+                CU_CHECK(p, launch_project_group(pg, b.B, b.R, !s.A32, st), "convert (band-limited)");
+            } else if (p->prec == TACAW_PREC_SPLIT_BF16)
                 CU_CHECK(p, launch_convert_split(gc, chunk, s.staged, p->bf, s.M_pad, s.mu_hat, s.sum_res, s.A_hi,
                                                  s.A_lo, 1, p->f16, p->f16_scale, p->d_err, st),
                          "convert");
@@ -1003,6 +1072,7 @@ tacaw_status finish_segment(tacaw_plan_s *p, UserStream &u, Stream &s, cudaStrea
     if (r != TACAW_OK) return r;
     CU_CHECK(p, cudaMemsetAsync(s.sum_res, 0, sizeof(double2) * s.M, st), "reset sums");
     s.pushed = s.staged = s.stage_start = s.flushes = 0;
+    s.form = -1;
     s.seg += u.lanes;
     return TACAW_OK;
 }
@@ -1305,6 +1375,15 @@ tacaw_status tacaw_plan_create(const tacaw_plan_desc *desc, tacaw_plan_t *out) {
         rc = build_stream(p, s, st);
         s.d.E_meV = nullptr;
     }
+    // band-limited staging forms, in what the budget leaves beside the staging and the frame tables
+    // (of whose 16 bytes an energy and frame `need` counts 4)
+    int64_t room = budget - need(K);
+    for (auto &s : p->s) room -= 12 * (int64_t)s.T_pad * s.Nw_pad;
+    for (size_t i = 0; i < p->s.size() && rc == TACAW_OK; ++i) {
+        const int64_t before = p->bytes;
+        rc = build_band_forms(p, p->s[i], room, st);
+        room -= p->bytes - before;
+    }
     for (auto &u : p->us) {
         if (rc != TACAW_OK) break;
         Stream &s0 = p->s[u.first];
@@ -1459,15 +1538,50 @@ tacaw_status tacaw_push_frames_group(tacaw_plan_t p, int n, const int *stream_id
     // pushes that fit their stream's ring as one tiled conversion go out together, the others
     // one by one as tacaw_push_frames does them
     std::vector<int> grouped;
+    std::vector<char> banded(n, 0);
     for (int i = 0; i < n; ++i) {
         const UserStream &u = p->us[stream_ids[i]];
-        const Stream &s = p->s[u.first];
+        Stream &s = p->s[u.first];
+        // pushes that lie in the ring and take one of its band-limited forms
+        if (u.N <= 1 && !p->in_place && !p->pipe && u.pushed >= u.skip && !s.due && s.staged + n_frames[i] <= s.ring) {
+            if (s.staged == 0) s.form = choose_form(p, s, n_frames[i]);
+            banded[i] = s.form >= 0;
+            if (banded[i]) continue;
+        }
         const bool ok = split && u.N <= 1 && u.pushed >= u.skip && !s.due && s.staged + n_frames[i] <= s.ring &&
                         convert_split_groupable(p->bf, s.staged, n_frames[i]);
         if (ok) {
             grouped.push_back(i);
         } else {
             c = push_user(p, stream_ids[i], static_cast<const float2 *>(d_frames[i]), n_frames[i], st);
+            if (c != TACAW_OK) return c;
+        }
+    }
+    // band-limited conversions: one launch for the streams on one basis
+    for (int i = 0; i < n; ++i) {
+        if (!banded[i]) continue;
+        const BandForm &b = p->s[p->us[stream_ids[i]].first].band[p->s[p->us[stream_ids[i]].first].form];
+        ProjGroup pg;
+        pg.n = 0;
+        std::copy(b.basis.begin(), b.basis.end(), pg.basis);
+        std::vector<int> ids;
+        for (int k = i; k < n && pg.n < kConvGroupMax; ++k) {
+            if (!banded[k]) continue;
+            Stream &s = p->s[p->us[stream_ids[k]].first];
+            if (s.band[s.form].B != b.B || s.band[s.form].R != b.R || s.band[s.form].beta != b.beta) continue;
+            banded[k] = 0;
+            ids.push_back(k);
+            const FrameGeom g = push_geom(s, static_cast<const float2 *>(d_frames[k]));
+            if (s.pushed == 0 && s.d.subtract_mean) {
+                CU_CHECK(p, launch_mean(g, n_frames[k], s.mu_hat, st), "provisional mean");
+                p->launches++;
+            }
+            pg.e[pg.n++] = proj_entry(p, s, g, n_frames[k]);
+        }
+        CU_CHECK(p, launch_project_group(pg, b.B, b.R, split, st), "convert (band-limited, group)");
+        p->launches++;
+        for (int k : ids) {
+            c = push_counted(p, p->us[stream_ids[k]], n_frames[k], st);
             if (c != TACAW_OK) return c;
         }
     }
@@ -1478,16 +1592,7 @@ tacaw_status tacaw_push_frames_group(tacaw_plan_t p, int n, const int *stream_id
             const int i = grouped[g0 + k];
             Stream &s = p->s[p->us[stream_ids[i]].first];
             ConvEntry &e = cg.e[k];
-            e.g.base = static_cast<const float2 *>(d_frames[i]);
-            e.g.pitch_row = s.d.pitch_row;
-            e.g.pitch_frame = s.d.pitch_frame;
-            e.g.pitch_probe = s.d.pitch_probe;
-            e.g.roi_x0 = s.d.roi_x0;
-            e.g.roi_y0 = s.d.roi_y0;
-            e.g.kx = s.d.kx;
-            e.g.ky = s.d.ky;
-            e.g.npix = s.npix;
-            e.g.M = s.M;
+            e.g = push_geom(s, static_cast<const float2 *>(d_frames[i]));
             e.n = n_frames[i];
             e.s0 = s.staged;
             e.M_pad = s.M_pad;
@@ -1504,15 +1609,8 @@ tacaw_status tacaw_push_frames_group(tacaw_plan_t p, int n, const int *stream_id
         p->launches++;
         for (int k = 0; k < cg.n; ++k) {
             const int i = grouped[g0 + k];
-            UserStream &u = p->us[stream_ids[i]];
-            Stream &s = p->s[u.first];
-            s.staged += n_frames[i];
-            s.pushed += n_frames[i];
-            u.pushed += n_frames[i];
-            if (s.staged == s.ring && s.pushed < s.T) {
-                s.due = true;     // deferrable: split, staged, one segment
-                s.due_stream = st;
-            }
+            c = push_counted(p, p->us[stream_ids[i]], n_frames[i], st);
+            if (c != TACAW_OK) return c;
         }
     }
     return TACAW_OK;
@@ -1603,6 +1701,7 @@ tacaw_status tacaw_reset(tacaw_plan_t p, void *stream) {
         CU_CHECK(p, cudaMemsetAsync(s.sum_res, 0, sizeof(double2) * s.M, st), "reset sums");
         CU_CHECK(p, cudaMemsetAsync(s.mu_hat, 0, sizeof(float2) * s.M, st), "reset mean");
         s.pushed = s.staged = s.stage_start = s.flushes = 0;
+        s.form = -1;
         s.seg = s.lane;
         s.due = false;
     }

@@ -277,6 +277,23 @@ cudaError_t launch_twiddles_fp32(const TableArgs &t, float2 *B32, cudaStream_t s
 cudaError_t launch_window_transform(const TableArgs &t, float2 *Wc, cudaStream_t st);
 cudaError_t launch_window_values(const TableArgs &t, float *w, cudaStream_t st);
 
+// Tables of the band-limited staging form: blocks of B frames, R coefficients, band centre fc (cycles
+// per frame).  basis [B/2][R] as in ProjGroup (FP64).
+struct BandTableArgs {
+    int B, R;
+    double fc;
+    const double *basis;
+    int ring;                  // frames per flush (a multiple of B, or >= T)
+    int slots;                 // table rows per flush (whole K-blocks of 32 on the split path)
+    int rounds;                // flushes a segment
+};
+cudaError_t launch_band_mod(const TableArgs &t, const BandTableArgs &b, float2 *mod, cudaStream_t st);
+// q_resp [R][Nw]: response of each basis vector at each energy (FP64; imaginary for the odd ones)
+cudaError_t launch_band_response(const TableArgs &t, const BandTableArgs &b, double *q_resp, cudaStream_t st);
+// split twiddles [rounds * slots / 32][2 Nw_pad][64] (pre-swizzled) or FP32 [rounds * slots][Nw_pad]
+cudaError_t launch_band_twiddles(const TableArgs &t, const BandTableArgs &b, const double *q_resp,
+                                 __nv_bfloat16 *B_hi, __nv_bfloat16 *B_lo, float2 *B32, cudaStream_t st);
+
 cudaError_t launch_mean(const FrameGeom &g, int n, float2 *mu_hat, cudaStream_t st);
 // f16 != 0: fp16 hi/lo pieces of f16_scale * (psi - mu_hat); a scaled component beyond the
 // fp16 range sets DEVERR_FP16_RANGE in *err
@@ -297,6 +314,38 @@ cudaError_t launch_zero_tail_split(int64_t M_pad, int staged, int bf, __nv_bfloa
 // dmu = scale * (mu - mu_hat) (scale: the split-FP16 operand scale, else 1)
 cudaError_t launch_mean_residual(int64_t M, int T, int subtract_mean, const double2 *sum_res, float2 *dmu,
                                  float scale, cudaStream_t st);
+
+// Push conversion into band-limited block coefficients (k_project.cu).  One push of one stream:
+struct ProjEntry {
+    FrameGeom g;
+    int n;                     // frames pushed
+    int c0;                    // frames of the current block already in the carry
+    int nblk;                  // blocks this push completes (with the segment's last frame also a short one)
+    int t_block;               // segment frame index of the first completed block's first frame
+    int slot0;                 // ring slot of its first coefficient (a multiple of 4)
+    int zero_slots;            // slots zeroed after the last block (a multiple of 4, up to the row's end)
+    int64_t M_pad;
+    const float2 *mu_hat;
+    double2 *sum_res;
+    float2 *carry;             // [B][M_pad] psi - mu_hat of an unfinished block
+    const float2 *mod;         // [T rounded up to B] window x shift to the band's centre, 0 past T
+    __nv_bfloat16 *A_hi, *A_lo;   // split staging (fp16 pieces), or
+    float2 *A32;                  // FP32 staging
+    float *row_scale;          // split staging: [M_pad] scale of the row's staged coefficients (0: all zero so far)
+    float f16_scale;           // split-FP16 plans: frames are checked against the fp16 range at this
+    uint32_t *err;             // scale (err not null)
+    int64_t group_begin;       // set by the launcher: first of its groups of 128 rows
+};
+struct ProjGroup {
+    ProjEntry e[kConvGroupMax];
+    int n;
+    int64_t groups;            // set by the launcher
+    alignas(16) float basis[64 * 48];   // [B/2][R] rows of the block's first half: R/2 even vectors, R/2 odd
+};
+// one launch over the pushes of pg.n <= kConvGroupMax streams, all on the same basis: blocks of B
+// frames, R coefficients (a shape project_shape_ok accepts), pg.basis; split: fp16 hi/lo rows of 32 slots, else FP32
+cudaError_t launch_project_group(ProjGroup &pg, int B, int R, bool split, cudaStream_t st);
+bool project_shape_ok(int B, int R, bool split);
 
 struct SimtArgs {
     EpiArgs e;
@@ -323,7 +372,9 @@ struct TcPlanArgs {
     int b_rows;                //   rows per twiddle block of B (2 * Nw_pad)
     int max_ctas;              // persistent grids: at most this many CTAs (0: one per SM)
     int N_last;                // staged form: columns of the last energy tile (<= N, multiple of 16)
-    int f16;                   // operands are fp16 pieces (split-FP16 path) instead of bf16
+    int f16;                   // operands are fp16 pieces (split-FP16 path, band-limited staging) instead of bf16
+    const float *row_scale;    // band-limited staging: [M_pad] power of two the row's coefficients are scaled by
+    float row_unit;            // (0: an empty row); its sums times row_unit / row_scale are the flush's result
     unsigned long long *trace; // null, or kTraceWords globaltimer stamps per CTA (phase boundaries)
     uint32_t *err;
     uint64_t wait_ns;          // pipeline waits give up after this many ns (0: the default 4 s)

@@ -15,6 +15,20 @@
 
 namespace tacaw {
 
+// A band-limited staging form of a stream (k_project.cu): blocks of B frames staged as R coefficients.
+struct BandForm {
+    int B = 0, R = 0;
+    double beta = 0.0;         // the band's width (with B and R: the basis)
+    int slots = 0;             // table rows per flush; the carry, then the row scales, follow
+                               // the ring's first `slots` slots
+    float2 *mod = nullptr;     // [T rounded up to B]
+    std::vector<float> basis;  // [B/2][R]
+    __nv_bfloat16 *B_hi = nullptr, *B_lo = nullptr;   // twiddles (split path)
+    float2 *B32 = nullptr;                            // twiddles (FP32 path)
+};
+constexpr int kBandForms = 2;
+constexpr int kBandDrainBlocks = 10;   // staging blocks per drained H chunk on band-limited forms
+
 struct Stream {
     tacaw_stream_desc d{};
     std::vector<double> E;
@@ -71,6 +85,28 @@ struct Stream {
                                                 // the stream at push time (no host copy)
     // segment state
     int pushed = 0, staged = 0, stage_start = 0, flushes = 0;
+    // staging forms besides the frames themselves; `form`: the one the ring holds now (its first push
+    // picks it: choose_form), -1: frames
+    BandForm band[kBandForms];
+    int n_band = 0;
+    int form = -1;
+    // staged slots of the ring: frames, or the coefficients of its blocks (whole ones, and at the
+    // segment's end a short one)
+    int ring_slots() const {
+        if (form < 0) return staged;
+        const BandForm &b = band[form];
+        return (pushed == T ? (staged + b.B - 1) / b.B : staged / b.B) * b.R;
+    }
+    // frames of an unfinished block, held in the carry
+    int carried() const { return form < 0 || pushed == T ? 0 : staged % band[form].B; }
+    float2 *carry() const {
+        const size_t o = (size_t)band[form].slots * (size_t)M_pad;
+        return A32 ? A32 + o : reinterpret_cast<float2 *>(A_hi + 2 * o);
+    }
+    // scales of the split form's rows: behind the carry
+    float *row_scale() const {
+        return A32 ? nullptr : reinterpret_cast<float *>(carry() + (size_t)band[form].B * (size_t)M_pad);
+    }
     // a full staging ring whose flush waits for the next push of this stream (or of finalize),
     // so that the flushes of several streams that fill up together share one launch
     bool due = false;
@@ -170,6 +206,11 @@ tacaw_status check_plan(tacaw_plan_s *p);
 tacaw_status check_kernel_memory(const void *ptr, const char *what, bool allow_host, cudaStream_t st);
 // Waits for `st` and turns the device error word into a status (poisoning the plan).
 tacaw_status read_device_error(tacaw_plan_s *p, cudaStream_t st);
+// Builds the band-limited staging forms that pay for stream s (tacaw_band.cu), within room_bytes of
+// device memory; a stream without any keeps staging frames.
+tacaw_status build_band_forms(tacaw_plan_s *p, Stream &s, int64_t room_bytes, cudaStream_t st);
+// The staging form a ring takes whose first push has n frames (-1: frames).
+int choose_form(const tacaw_plan_s *p, const Stream &s, int n);
 // Table arguments of stream s after its tables were built.
 TableArgs stream_table_args(const Stream &s, int block_frames);
 

@@ -36,7 +36,8 @@ struct StateHeader {
 };
 struct StreamCounters {
     int64_t pushed, staged, stage_start, flushes, seg;
-    int32_t due, reserved;
+    int32_t due;
+    int32_t form;             // staging form of the ring: 0 frames, else the block length B of its band-limited form
 };
 struct UserCounters {
     int64_t pushed;
@@ -115,6 +116,13 @@ struct StateSection {
     size_t bytes;
 };
 
+// Index of stream s's band-limited form with blocks of B frames (-1: frames, or no such form).
+int band_of(const Stream &s, int B) {
+    for (int i = 0; i < s.n_band; ++i)
+        if (s.band[i].B == B) return i;
+    return -1;
+}
+
 // Device sections of a checkpoint whose streams have the counters c, in checkpoint order.
 std::vector<StateSection> state_sections(const tacaw_plan_s *p, const std::vector<StreamCounters> &c) {
     std::vector<StateSection> v;
@@ -124,15 +132,28 @@ std::vector<StateSection> state_sections(const tacaw_plan_s *p, const std::vecto
         v.push_back({s.sum_res, sizeof(double2) * (size_t)s.M});
         if (c[i].staged > 0) {
             // staged frames fill ring slots [0, staged): whole blocks of bf frames (split) or
-            // frame-major rows of M_pad (FP32)
+            // frame-major rows of M_pad (FP32); a band-limited form's whole blocks fill B / R as many,
+            // the frames of an unfinished block its carry
+            Stream k;              // the ring as the counters describe it
+            k.form = band_of(s, c[i].form);
+            k.pushed = (int)c[i].pushed;
+            k.staged = (int)c[i].staged;
+            k.T = s.T;
+            k.M_pad = s.M_pad;
+            k.A_hi = s.A_hi;
+            k.A32 = s.A32;
+            if (k.form >= 0) k.band[k.form] = s.band[k.form];
+            const int64_t slots = k.ring_slots();
             if (p->prec == TACAW_PREC_SPLIT_BF16) {
-                const size_t n = (size_t)((c[i].staged + p->bf - 1) / p->bf) * (size_t)s.M_pad * 2 * p->bf *
+                const size_t n = (size_t)((slots + p->bf - 1) / p->bf) * (size_t)s.M_pad * 2 * p->bf *
                                  sizeof(__nv_bfloat16);
                 v.push_back({s.A_hi, n});
                 v.push_back({s.A_lo, n});
             } else {
-                v.push_back({s.A32, sizeof(float2) * (size_t)c[i].staged * (size_t)s.M_pad});
+                v.push_back({s.A32, sizeof(float2) * (size_t)slots * (size_t)s.M_pad});
             }
+            if (k.form >= 0 && slots > 0 && !s.A32) v.push_back({k.row_scale(), sizeof(float) * (size_t)s.M_pad});
+            if (k.carried()) v.push_back({k.carry(), sizeof(float2) * (size_t)k.carried() * (size_t)s.M_pad});
         }
         if (s.needs_acc && c[i].flushes > 0) {
             const size_t n = (size_t)s.Nw * (size_t)s.M_pad;   // energies j < Nw, rows of M_pad
@@ -150,7 +171,8 @@ std::vector<StreamCounters> plan_counters(const tacaw_plan_s *p) {
     std::vector<StreamCounters> c(p->s.size());
     for (size_t i = 0; i < p->s.size(); ++i) {
         const Stream &s = p->s[i];
-        c[i] = StreamCounters{s.pushed, s.staged, s.stage_start, s.flushes, s.seg, s.due ? 1 : 0, 0};
+        c[i] = StreamCounters{s.pushed, s.staged, s.stage_start, s.flushes, s.seg, s.due ? 1 : 0,
+                              s.form >= 0 ? s.band[s.form].B : 0};
     }
     return c;
 }
@@ -200,6 +222,7 @@ tacaw_status check_counters(const tacaw_plan_s *p, const std::vector<StreamCount
                         k.stage_start >= 0 && k.stage_start + k.staged == k.pushed && k.flushes >= 0 &&
                         k.flushes <= k.stage_start && (s.needs_acc || k.flushes == 0) &&
                         (!p->in_place || k.staged == 0) && (k.due == 0 || (k.due == 1 && k.staged == s.ring)) &&
+                        (k.form == 0 || (k.staged > 0 && band_of(s, k.form) >= 0)) &&
                         k.seg >= s.lane && (k.seg - s.lane) % u.lanes == 0 &&
                         k.seg < s.lane + (int64_t)u.lanes * (u.N + 1);
         if (!ok) return fail(TACAW_ERR_INVALID_ARG, "checkpoint: counters of stream %zu are inconsistent", i);
@@ -318,6 +341,7 @@ tacaw_status tacaw_restore_state(tacaw_plan_t p, const void *h_state, int64_t by
         s.staged = (int)cnt[i].staged;
         s.stage_start = (int)cnt[i].stage_start;
         s.flushes = (int)cnt[i].flushes;
+        s.form = band_of(s, cnt[i].form);
         s.seg = cnt[i].seg;
         s.due = cnt[i].due != 0;
         s.due_stream = st;
