@@ -252,7 +252,7 @@ __device__ __forceinline__ void split2_bf16(float2 r, uint32_t &hi, uint32_t &lo
 // Drained form: per-thread FP32 running sums of up to kDrainCols accumulator columns (one TMEM
 // lane, a contiguous column range: tiles of at most 112 complex energies).  Loads are
 // warp-uniform; columns past `cols` (up to 15 of them, inside the allocation) are loaded and
-// ignored.
+// added into sums nobody reads.
 constexpr int kDrainCols = 112;
 template <int C>
 __device__ __forceinline__ void drain_add(float (&sum)[C], uint32_t taddr, int cols) {
@@ -264,7 +264,7 @@ __device__ __forceinline__ void drain_add(float (&sum)[C], uint32_t taddr, int c
             tmem_ld_wait();
 #pragma unroll
             for (int i = 0; i < 16; ++i)
-                if (r * 16 + i < C && r * 16 + i < cols) sum[r * 16 + i] += __uint_as_float(x[i]);
+                if (r * 16 + i < C) sum[r * 16 + i] += __uint_as_float(x[i]);
         }
         __syncwarp();
     }
@@ -300,6 +300,47 @@ __device__ __forceinline__ void tc_epilogue_prefetch(const TcPlanArgs &a, int64_
         }
         if (acc64) prefetch_l2(e.acc_d + ai);
         if (iadd) prefetch_l2(e.I_out + o0 + (int64_t)j * e.npix);
+    }
+}
+
+// The same for the epilogues that only store, one output to a row and energy: I stored (OUT 0) or added
+// to (1), Psi alone (2), plain FP32 accumulators (3).  The general form above reads its arguments and
+// forms its addresses anew at every element (the 112 sums leave no registers to keep them): 4750 warp
+// instructions a 104-energy tile, 15 us, which tiles of up to a dozen staging blocks wait for.  Here the
+// output pointer advances by one pitch an energy and the tables are read at constant offsets.
+template <int OUT, int C>
+__device__ __forceinline__ void tc_epilogue_store(const TcPlanArgs &a, const RowCtx &row, int col0, int cols, int jbase,
+                                                  const float (&sum)[C]) {
+    if (!row.valid) return;
+    const EpiArgs &e = a.e;
+    const int j0 = jbase + (col0 >> 1), n = min(cols >> 1, e.Nw - j0);
+    const float2 *W = e.Wc + j0;
+    const float *B = e.bose + j0;
+    const float scale = OUT == 2 ? e.psi_scale : e.out_scale;
+    const int64_t pitch = OUT == 3 ? e.M_pad : e.npix;
+    const int64_t o = OUT == 3 ? (int64_t)j0 * pitch + row.m : row.out_base + (int64_t)j0 * pitch;
+    float *I = e.I_out + o;
+    float2 *P = (OUT == 3 ? e.acc_s : e.Psi_out) + o;
+#pragma unroll
+    for (int i = 0; i < C / 2; ++i) {
+        if (i >= n) break;
+        float pr = sum[2 * i], pi = sum[2 * i + 1];
+        if (OUT == 3) {
+            *P = make_float2(pr, pi);
+            P += pitch;
+            continue;
+        }
+        const float2 w = __ldg(W + i);
+        pr -= row.dmu.x * w.x - row.dmu.y * w.y;
+        pi -= row.dmu.x * w.y + row.dmu.y * w.x;
+        if (OUT == 2) {
+            *P = make_float2(pr * scale, pi * scale);
+            P += pitch;
+        } else {
+            const float v = (pr * pr + pi * pi) * __ldg(B + i) * scale;
+            *I = OUT == 1 ? *I + v : v;
+            I += pitch;
+        }
     }
 }
 
@@ -700,13 +741,19 @@ __global__ void __maxnreg__(168) flush_tc_drain2_kernel(const __grid_constant__ 
                 const int64_t mrow = (int64_t)m0 + q4 * 32 + lane;
                 const int j0 = wtile * a.wt + (col0 >> 1);
                 const int nv = (preload && mrow < a.e.M) ? max(0, min(cols >> 1, a.e.Nw - j0)) : 0;
-                const float2 *ap = preload ? a.e.acc_s + (size_t)j0 * (size_t)a.e.M_pad + (size_t)mrow : nullptr;
-                const size_t stride = (size_t)a.e.M_pad;
+                if (preload) {
+                    const float2 *ap = a.e.acc_s + (size_t)j0 * (size_t)a.e.M_pad + (size_t)mrow;
+                    const size_t stride = (size_t)a.e.M_pad;
 #pragma unroll
-                for (int i = 0; i < kDrainCols / 2; ++i) {
-                    const float2 v = i < nv ? ap[(size_t)i * stride] : make_float2(0.f, 0.f);
-                    sum[2 * i] = v.x;
-                    sum[2 * i + 1] = v.y;
+                    for (int i = 0; i < kDrainCols / 2; ++i) {
+                        const float2 v = i < nv ? *ap : make_float2(0.f, 0.f);
+                        ap += stride;
+                        sum[2 * i] = v.x;
+                        sum[2 * i + 1] = v.y;
+                    }
+                } else {
+#pragma unroll
+                    for (int i = 0; i < kDrainCols; ++i) sum[i] = 0.f;
                 }
                 if (BAND && preload && a.row_scale) {
                     const float ps = 1.f / row_factor(a, mrow);
@@ -751,6 +798,20 @@ __global__ void __maxnreg__(168) flush_tc_drain2_kernel(const __grid_constant__ 
             // with preloaded sums an update of the accumulators is a store, a finalize one without
             // earlier flushes
             const int kind = preload ? (kind0 == EPI_ADD_KAHAN ? EPI_STORE_KAHAN : EPI_FINAL) : kind0;
+            if (kind == EPI_FINAL && !a.e.Psi_out) {
+                if (!a.e.I_out) continue;
+                if (a.e.out_add) tc_epilogue_store<1>(a, row, col0, cols, jbase, sum);
+                else tc_epilogue_store<0>(a, row, col0, cols, jbase, sum);
+                continue;
+            }
+            if (kind == EPI_FINAL && !a.e.I_out) {
+                tc_epilogue_store<2>(a, row, col0, cols, jbase, sum);
+                continue;
+            }
+            if (kind == EPI_STORE_KAHAN && !a.e.acc_c) {
+                tc_epilogue_store<3>(a, row, col0, cols, jbase, sum);
+                continue;
+            }
             switch (kind) {
                 case EPI_FINAL: tc_epilogue_regs<EPI_FINAL>(a, row, col0, cols, jbase, sum); break;
                 case EPI_FINAL_KAHAN: tc_epilogue_regs<EPI_FINAL_KAHAN>(a, row, col0, cols, jbase, sum); break;

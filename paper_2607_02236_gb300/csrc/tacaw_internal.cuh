@@ -99,8 +99,9 @@ __device__ __forceinline__ RowCtx make_row(const EpiArgs &a, int64_t m) {
     RowCtx r;
     r.m = m;
     r.valid = m < a.M;
-    int64_t p = r.valid ? m / a.npix : 0;
-    int64_t pix = m - p * a.npix;
+    // (rows fit 32 bits, checked at plan creation: a 64-bit division is several times as long)
+    const int64_t p = r.valid ? (int64_t)((uint32_t)m / (uint32_t)a.npix) : 0;
+    const int64_t pix = m - p * a.npix;
     r.out_base = p * (int64_t)a.Nw * a.npix + pix;
     r.dmu = (r.valid && a.dmu) ? a.dmu[m] : make_float2(0.f, 0.f);
     return r;
