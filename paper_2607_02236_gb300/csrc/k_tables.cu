@@ -242,7 +242,7 @@ __global__ void band_mod_kernel(TableArgs a, int B, double fc, int n, float2 *mo
 __global__ void band_response_kernel(TableArgs a, BandTableArgs b, double *q_resp) {
     const int j = blockIdx.x * blockDim.x + threadIdx.x, q = blockIdx.y;
     if (j >= a.Nw) return;
-    const double d = a.cj[j] - b.fc;
+    const double d = a.cj[j] - (b.fcj ? b.fcj[j] : b.fc);
     double acc = 0.0;
     for (int u = 0; u < b.B / 2; ++u) {
         double c, s;
@@ -302,6 +302,55 @@ __global__ void band_twiddles_kernel(TableArgs a, BandTableArgs b, const double 
             B_lo[r1 + e] = l;
         }
     }
+}
+
+// Second-level coefficient p of energy group g over a superblock: sum_t x_t w_p[t] exp(-2 pi i f_g (t - (S-1)/2)),
+// x_t = exp(2 pi i f_c (u - c)) sum_q z[k, q] v_q[u] for t = k B + u.  One thread per (column g r + p, slot k R + q).
+__global__ void band_merge_kernel(BandMergeArgs m, __nv_bfloat16 *T_hi, __nv_bfloat16 *T_lo) {
+    const int col = blockIdx.x * blockDim.x + threadIdx.x, slot = blockIdx.y * blockDim.y + threadIdx.y;
+    const int B = m.b.B, R = m.b.R;
+    if (col >= m.cols_pad || slot >= m.S / B * R) return;
+    double ar = 0.0, ai = 0.0;
+    if (col < m.groups * m.r) {
+        const int g = col / m.r, p = col % m.r, k = slot / R, q = slot % R;
+        const double fg = m.fg[g], c0 = 0.5 * (double)(B - 1);
+        const bool odd_v = q >= R / 2, odd_w = p >= m.r / 2;
+        double sr = 0.0, si = 0.0;
+        for (int u = 0; u < B; ++u) {
+            const double v = u < B / 2 ? m.b.basis[u * R + q] : (odd_v ? -1.0 : 1.0) * m.b.basis[(B - 1 - u) * R + q];
+            const int t = k * B + u;
+            const double w = t < m.S / 2 ? m.w[t * m.r + p] : (odd_w ? -1.0 : 1.0) * m.w[(m.S - 1 - t) * m.r + p];
+            double s, c;
+            sincospi(2.0 * (m.b.fc - fg) * ((double)u - c0), &s, &c);
+            sr += v * w * c;
+            si += v * w * s;
+        }
+        double s, c;
+        sincospi(-2.0 * fg * ((double)(k * B) + c0 - 0.5 * (double)(m.S - 1)), &s, &c);
+        ar = sr * c - si * s;
+        ai = sr * s + si * c;
+    }
+    const int kb = slot / 32, tt = slot % 32, n0 = 2 * col, n1 = 2 * col + 1;
+    const int w0 = (((tt >> 2) ^ (n0 & 7)) << 2) | (tt & 3), w1 = (((tt >> 2) ^ (n1 & 7)) << 2) | (tt & 3);
+    const size_t rows = 2 * (size_t)m.cols_pad;
+    const size_t r0 = ((size_t)kb * rows + (size_t)n0) * 64 + 2 * (size_t)w0;
+    const size_t r1 = ((size_t)kb * rows + (size_t)n1) * 64 + 2 * (size_t)w1;
+    const float v0[2] = {(float)ar, (float)(-ai)}, v1[2] = {(float)ai, (float)ar};
+    for (int e = 0; e < 2; ++e) {
+        __nv_bfloat16 h, l;
+        split_f16(v0[e], h, l);
+        T_hi[r0 + e] = h;
+        T_lo[r0 + e] = l;
+        split_f16(v1[e], h, l);
+        T_hi[r1 + e] = h;
+        T_lo[r1 + e] = l;
+    }
+}
+
+cudaError_t launch_band_merge(const BandMergeArgs &m, __nv_bfloat16 *T_hi, __nv_bfloat16 *T_lo, cudaStream_t st) {
+    const int slots = m.S / m.b.B * m.b.R;
+    band_merge_kernel<<<dim3((m.cols_pad + 31) / 32, (slots + 3) / 4), dim3(32, 4), 0, st>>>(m, T_hi, T_lo);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_band_mod(const TableArgs &t, const BandTableArgs &b, float2 *mod, cudaStream_t st) {

@@ -350,6 +350,71 @@ __device__ __forceinline__ float row_factor(const TcPlanArgs &a, int64_t m) {
     return a.row_unit / (s == 0.f ? 1.f : s);
 }
 
+// Superblock of local tile lt, and its staging blocks (the last superblock may be short).
+__device__ __forceinline__ int tc_superblock(const TcPlanArgs &a, int64_t lt) {
+    return a.n_sb > 1 ? (int)(lt / a.n_wt % a.n_sb) : 0;
+}
+__device__ __forceinline__ int tc_blocks(const TcPlanArgs &a, int sb) {
+    return a.n_sb > 0 ? min(a.n_kb, a.total_kb - sb * a.n_kb) : a.n_kb;
+}
+
+// First level of a two-level contraction: the columns [c0, c0 + n) of superblock sb of row m as fp16 hi + lo
+// of their group's staged rows; n, c0 and z_r are multiples of 8, so eight columns lie in one group and
+// fill one 32-byte sector of its row (two chunks, which the swizzle exchanges but does not part), stored
+// whole: 16-byte stores took 1.6 of the 4.4 ms of the thick case's first level.  The last
+// superblock's last column zeroes the rest of its 32-slot row.
+__device__ __forceinline__ void st_sector(uint4 *p, const uint32_t (&v)[8], bool swap) {
+    const int x = swap ? 4 : 0;
+    uint32_t w[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) w[k] = x ? v[k ^ 4] : v[k];
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(w[0]), "r"(w[1]), "r"(w[2]),
+                 "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
+                 : "memory");
+}
+template <int C>
+__device__ __forceinline__ void tc_store_z(const TcPlanArgs &a, int64_t m, int sb, int c0, int n,
+                                           const float (&sum)[C]) {
+    const int sw = (int)(m & 7), zr = a.z_r, n_in = min(n, a.z_cols - c0);
+    const int64_t pitch = a.e.M_pad * 8;                       // chunks from a 32-slot row to the next
+    const int64_t group = (int64_t)(a.z_slots >> 5) * pitch;
+    const bool tail = sb == a.n_sb - 1;
+    const float mul = a.z_mul;
+    int q = c0 % zr;
+    uint4 *hi = static_cast<uint4 *>(a.z_hi) + (c0 / zr) * group + m * 8;
+    uint4 *lo = static_cast<uint4 *>(a.z_lo) + (c0 / zr) * group + m * 8;
+#pragma unroll
+    for (int i = 0; i < C / 2; i += 8) {
+        if (i >= n_in) break;
+        uint32_t h[8], l[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const float2 v = make_float2(sum[2 * (i + k)] * mul, sum[2 * (i + k) + 1] * mul);
+            const __half2 p = __float22half2_rn(v);
+            const float2 b = __half22float2(p);
+            const __half2 d = __floats2half2_rn(v.x - b.x, v.y - b.y);
+            memcpy(&h[k], &p, 4);
+            memcpy(&l[k], &d, 4);
+        }
+        int ch = (sb * zr + q) >> 2;                           // even: chunks ch, ch + 1 in one sector
+        int64_t o = (int64_t)(ch >> 3) * pitch + (((ch & 7) ^ sw) & ~1);
+        st_sector(hi + o, h, sw & 1);
+        st_sector(lo + o, l, sw & 1);
+        q += 8;
+        if (q == zr) {
+            if (tail)
+                for (ch += 2; ch & 7; ++ch) {
+                    o = (int64_t)(ch >> 3) * pitch + ((ch & 7) ^ sw);
+                    hi[o] = make_uint4(0, 0, 0, 0);
+                    lo[o] = make_uint4(0, 0, 0, 0);
+                }
+            q = 0;
+            hi += group;
+            lo += group;
+        }
+    }
+}
+
 // Flush epilogue of the split drained form: the tile's result is all in the running sums.
 template <int KIND, int C>
 __device__ __forceinline__ void tc_epilogue_regs(const TcPlanArgs &a, const RowCtx &row, int col0, int cols,
@@ -554,7 +619,9 @@ __global__ void __maxnreg__(168) flush_tc_drain2_kernel(const __grid_constant__ 
                 const TcGroupEntry &en = g.e[gi];
                 const int64_t lt = t - en.cta_begin;
                 const int wtile = (int)(lt % en.args.n_wt);
-                const int m0 = (int)(lt / en.args.n_wt) * kMTile;
+                const int sb = BAND ? tc_superblock(en.args, lt) : 0;
+                const int m0 = (int)(lt / en.args.n_wt / (BAND ? max(1, en.args.n_sb) : 1)) * kMTile;
+                const int n_kb = BAND ? tc_blocks(en.args, sb) : en.args.n_kb;
                 const int N = en.args.N;
                 // columns of this tile (N_last: a narrower last energy tile; 0 = full width)
                 const int Nt = (wtile == en.args.n_wt - 1 && en.args.N_last > 0) ? en.args.N_last : N;
@@ -565,7 +632,12 @@ __global__ void __maxnreg__(168) flush_tc_drain2_kernel(const __grid_constant__ 
                 const uint8_t *pBhi = static_cast<const uint8_t *>(en.args.B_hi) + b0;
                 const uint8_t *pBlo = static_cast<const uint8_t *>(en.args.B_lo) + b0;
                 const size_t a_step = (size_t)en.args.a_rows * RB, b_step = (size_t)en.args.b_rows * RB;
-                for (int kb = 0; kb < en.args.n_kb; ++kb) {
+                if (BAND) {
+                    const size_t off = (size_t)sb * (size_t)en.args.n_kb * a_step + (size_t)wtile * (size_t)en.args.a_group;
+                    pAhi += off;
+                    pAlo += off;
+                }
+                for (int kb = 0; kb < n_kb; ++kb) {
                     if (!mbar_wait(smem_u32(&sh->empty[s]), ph ^ 1u, abort_flag, wait_ns)) {
                         if (!*abort_flag) atomicOr(err, DEVERR_TIMEOUT_EMPTY);
                         *abort_flag = 1;
@@ -630,7 +702,8 @@ __global__ void __maxnreg__(168) flush_tc_drain2_kernel(const __grid_constant__ 
                 if (t < 0) break;
                 const TcGroupEntry &en = g.e[group_entry(g, t)];
                 const bool last_w = en.args.N_last > 0 && (t - en.cta_begin) % en.args.n_wt == en.args.n_wt - 1;
-                const int N = last_w ? en.args.N_last : en.args.N, n_kb = en.args.n_kb, cb = en.args.drain_kb;
+                const int N = last_w ? en.args.N_last : en.args.N, cb = en.args.drain_kb;
+                const int n_kb = BAND ? tc_blocks(en.args, tc_superblock(en.args, t - en.cta_begin)) : en.args.n_kb;
                 const uint32_t id = idesc_f32acc(kMTile, N, en.args.f16);
                 if (tiles > 0) {
                     // the previous tile's H and S must be in registers before they are reused
@@ -725,12 +798,13 @@ __global__ void __maxnreg__(168) flush_tc_drain2_kernel(const __grid_constant__ 
             const TcPlanArgs &a = en.args;
             const int64_t lt = t - en.cta_begin;
             const int wtile = (int)(lt % a.n_wt);
-            const int m0 = (int)(lt / a.n_wt) * kMTile;
+            const int sb = BAND ? tc_superblock(a, lt) : 0;
+            const int m0 = (int)(lt / a.n_wt / (BAND ? max(1, a.n_sb) : 1)) * kMTile;
             // N / 2 columns per thread (the last energy tile may be narrower)
             const int cols = ((wtile == a.n_wt - 1 && a.N_last > 0) ? a.N_last : a.N) / 2;
             const int col0 = h * cols;
             const uint32_t lane_base = tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)col0;
-            const int n_chunks = (a.n_kb + a.drain_kb - 1) / a.drain_kb;
+            const int n_chunks = ((BAND ? tc_blocks(a, sb) : a.n_kb) + a.drain_kb - 1) / a.drain_kb;
             // plain FP32 accumulators of earlier flushes start this tile's running sums: read while
             // the tile's first products run, so that the tile's epilogue only stores (the reads
             // then wait on nothing); compensated and FP64 accumulators are added at the end
@@ -788,6 +862,10 @@ __global__ void __maxnreg__(168) flush_tc_drain2_kernel(const __grid_constant__ 
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&sh->chunk_free[1]));
+            if (BAND && a.z_hi) {
+                tc_store_z(a, (int64_t)m0 + q4 * 32 + lane, sb, wtile * a.wt + (col0 >> 1), cols >> 1, sum);
+                continue;
+            }
             const RowCtx row = make_row(a.e, (int64_t)m0 + q4 * 32 + lane);
             const int jbase = wtile * a.wt;
             if (BAND && a.row_scale) {
@@ -1488,7 +1566,7 @@ int tc_resident_ctas(int N, int bf, int stages) {
     return n * sms;
 }
 
-int64_t tc_grid_ctas(const TcPlanArgs &a) { return a.e.M_pad / kMTile * a.n_wt; }
+int64_t tc_grid_ctas(const TcPlanArgs &a) { return a.e.M_pad / kMTile * a.n_wt * std::max(1, a.n_sb); }
 
 static cudaError_t launch_flush_tc_group_impl(const TcPlanArgs *args, int n, const TcConvJob *conv,
                                               cudaStream_t st) {
@@ -1526,7 +1604,7 @@ static cudaError_t launch_flush_tc_group_impl(const TcPlanArgs *args, int n, con
     g->tiles = total;
     const size_t smem = tc_smem_bytes(n_max, args[0].bf, g->stages);
     bool band = false;
-    for (int i = 0; i < n; ++i) band = band || args[i].row_scale;
+    for (int i = 0; i < n; ++i) band = band || args[i].row_scale || args[i].z_hi;
     void (*kern)(TcGroup) = band ? flush_tc_drain2_kernel<true> : flush_tc_drain2_kernel<false>;
     int dev = 0, sms = 0, occ = 0;
     cudaError_t e = cudaGetDevice(&dev);

@@ -259,9 +259,67 @@ TcPlanArgs tc_args(tacaw_plan_s *p, const Stream &s, const EpiArgs &e) {
     a.f16 = band || p->f16;
     a.row_scale = band ? s.row_scale() : nullptr;
     a.row_unit = p->f16_scale;
+    if (band && band->S) {
+        // second level: each energy tile over its own group's coefficients
+        const int n_sb = (a.n_kb * p->bf + band->S / band->B * band->R - 1) / (band->S / band->B * band->R);
+        a.n_kb = (n_sb * band->r + p->bf - 1) / p->bf;
+        a.kbB0 = s.stage_start / s.ring * (band->z_slots / p->bf);
+        a.A_hi = s.A_hi + 2 * (size_t)band->z_begin() * (size_t)s.M_pad;
+        a.A_lo = s.A_lo + 2 * (size_t)band->z_begin() * (size_t)s.M_pad;
+        a.a_group = 4 * (int64_t)band->z_slots * s.M_pad;
+        a.row_unit *= (float)(1 << band->z_shift());
+        a.drain_kb = std::min(a.drain_kb, 4);   // (the first level's sums are truncated too)
+    }
     a.err = p->d_err;
     a.trace = nullptr;
     return a;
+}
+
+// Two-level contractions: the first level of the flushes of streams ids, in one launch.
+tacaw_status launch_first_level(tacaw_plan_s *p, const Stream *const *streams, int n, cudaStream_t st) {
+    std::vector<TcPlanArgs> args;
+    for (int i = 0; i < n; ++i) {
+        const Stream &s = *streams[i];
+        if (s.form < 0 || !s.band[s.form].S) continue;
+        const BandForm &b = s.band[s.form];
+        TcPlanArgs a{};
+        a.e.M = s.M;
+        a.e.M_pad = s.M_pad;
+        a.e.npix = s.npix;
+        a.e.mode = FLUSH_FINAL;
+        a.wt = b.wt1;
+        a.n_wt = b.n_wt1;
+        a.N = 2 * b.wt1;
+        a.z_cols = s.n_wt * b.r;
+        a.N_last = std::min(a.N, (int)round_up(2 * (a.z_cols - (b.n_wt1 - 1) * b.wt1), 32));   // whole sectors a thread
+        a.total_kb = (s.ring_slots() + p->bf - 1) / p->bf;
+        a.n_kb = b.S / b.B * b.R / p->bf;
+        a.n_sb = (a.total_kb + a.n_kb - 1) / a.n_kb;
+        a.bf = p->bf;
+        a.stages = s.stages;
+        a.drain_kb = kBandDrainBlocks;
+        a.A_hi = s.A_hi;
+        a.A_lo = s.A_lo;
+        a.B_hi = b.T_hi;
+        a.B_lo = b.T_lo;
+        a.a_rows = s.M_pad;
+        a.b_rows = 2 * b.wt1 * b.n_wt1;
+        a.max_ctas = p->tc_max_ctas;
+        a.wait_ns = p->wait_ns;
+        a.f16 = 1;
+        a.err = p->d_err;
+        a.z_hi = s.A_hi + 2 * (size_t)b.z_begin() * (size_t)s.M_pad;
+        a.z_lo = s.A_lo + 2 * (size_t)b.z_begin() * (size_t)s.M_pad;
+        a.z_r = b.r;
+        a.z_slots = b.z_slots;
+        a.z_mul = 1.f / (float)(1 << b.z_shift());
+        args.push_back(a);
+    }
+    if (args.empty()) return TACAW_OK;
+    args[0].tile_counter = p->d_counters + (p->counter_slot++ % kCounterRing);
+    CU_CHECK(p, launch_flush_tc_group(args.data(), (int)args.size(), st), "flush (first level)");
+    p->launches++;
+    return TACAW_OK;
 }
 
 // Per-CTA phase trace of the next flush launch (nc CTAs).
@@ -372,6 +430,9 @@ tacaw_status run_flush(tacaw_plan_s *p, Stream &s, int mode, float *I_out, float
             CU_CHECK(p, launch_zero_tail_split(s.M_pad, n, p->bf, s.A_hi, s.A_lo, 1, st), "zero_tail");
             p->launches++;
         }
+        const Stream *one = &s;
+        r = launch_first_level(p, &one, 1, st);
+        if (r != TACAW_OK) return r;
         TcPlanArgs a = tc_args(p, s, e);
         a.tile_counter = p->d_counters + (p->counter_slot++ % kCounterRing);
         r = trace_buffer(p, tc_grid_ctas(a), &a.trace);
@@ -436,6 +497,10 @@ tacaw_status flush_grouped(tacaw_plan_s *p, std::vector<FlushReq> req, cudaStrea
         args[0].tile_counter = p->d_counters + (p->counter_slot++ % kCounterRing);
         cudaEvent_t e0, e1;
         r = timing_begin(p, &e0, &e1, st);
+        if (r != TACAW_OK) return r;
+        std::vector<const Stream *> group;
+        for (size_t k = g0; k < g1; ++k) group.push_back(&p->s[req[k].s]);
+        r = launch_first_level(p, group.data(), (int)group.size(), st);
         if (r != TACAW_OK) return r;
         CU_CHECK(p, launch_flush_tc_group(args.data(), (int)args.size(), st), "flush (tensor cores, grouped)");
         p->launches++;
@@ -785,6 +850,9 @@ tacaw_status launch_pending(tacaw_plan_s *p, const Stream *conv, cudaStream_t st
     if (r != TACAW_OK) return r;
     cudaEvent_t e0, e1;
     r = timing_begin(p, &e0, &e1, st);
+    if (r != TACAW_OK) return r;
+    const Stream *one = &ps;
+    r = launch_first_level(p, &one, 1, st);
     if (r != TACAW_OK) return r;
     if (conv) {
         TcConvJob j{};
@@ -1378,10 +1446,11 @@ tacaw_status tacaw_plan_create(const tacaw_plan_desc *desc, tacaw_plan_t *out) {
     // band-limited staging forms, in what the budget leaves beside the staging and the frame tables
     // (of whose 16 bytes an energy and frame `need` counts 4)
     int64_t room = budget - need(K);
+    BandCache bases;
     for (auto &s : p->s) room -= 12 * (int64_t)s.T_pad * s.Nw_pad;
     for (size_t i = 0; i < p->s.size() && rc == TACAW_OK; ++i) {
         const int64_t before = p->bytes;
-        rc = build_band_forms(p, p->s[i], room, st);
+        rc = build_band_forms(p, p->s[i], room, bases, st);
         room -= p->bytes - before;
     }
     for (auto &u : p->us) {

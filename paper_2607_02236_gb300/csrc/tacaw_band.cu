@@ -35,40 +35,49 @@ public:
             hi = std::max(hi, d[u] + r);
         }
     }
-    // the k-th sequence's first half, the whole sequence of unit norm (norm sqrt(1/2))
-    std::vector<double> vector(int k) const {
-        double a = lo, b = hi;   // the k-th largest eigenvalue
-        for (int i = 0; i < 80 && b - a > 4e-16 * std::max(std::fabs(a), std::fabs(b)); ++i) {
-            const double x = 0.5 * (a + b);
-            (above(x) > k ? a : b) = x;
+    // first halves of the n most concentrated sequences, the whole sequences of unit norm (norm sqrt(1/2))
+    std::vector<std::vector<double>> vectors(int n) const {
+        n = std::min(n, H);
+        // all eigenvalues side by side: each count is a chain of divisions, which the others overlap
+        std::vector<double> a(n, lo), b(n, hi), q(n), x(n);
+        std::vector<int> above(n);
+        for (int i = 0; i < 32; ++i) {   // to 2^-32 of the range, far below the gaps (about range / B^2)
+            for (int k = 0; k < n; ++k) {
+                x[k] = 0.5 * (a[k] + b[k]);
+                q[k] = 1.0;
+                above[k] = 0;
+            }
+            for (int u = 0; u < H; ++u) {
+                const double o2 = o[u] * o[u];   // (o[0] = 0)
+                for (int k = 0; k < n; ++k) {
+                    double t = d[u] - x[k] - o2 / q[k];
+                    t = t == 0.0 ? 1e-300 : t;
+                    above[k] += t > 0.0;         // positive pivots of A - x: eigenvalues above x
+                    q[k] = t;
+                }
+            }
+            for (int k = 0; k < n; ++k) (above[k] > k ? a[k] : b[k]) = x[k];
         }
-        const double x = 0.5 * (a + b) + 1e-13 * (hi - lo);   // off the eigenvalue: the solves stay finite
-        std::vector<double> v(H, 1.0);
-        for (int u = 0; u < H; ++u) v[u] += 0.01 * (u % 7);   // no symmetry that could hide a vector
-        for (int it = 0; it < 4; ++it) {
-            solve(x, v);
-            double n = 0.0;
-            for (double t : v) n += t * t;
-            for (double &t : v) t *= std::sqrt(0.5 / n);
+        std::vector<std::vector<double>> out;
+        for (int k = 0; k < n; ++k) {
+            const double shift = 0.5 * (a[k] + b[k]) + 1e-11 * (hi - lo);   // off the eigenvalue: the solves stay finite
+            std::vector<double> v(H);
+            for (int u = 0; u < H; ++u) v[u] = 1.0 + 0.01 * (u % 7);   // no symmetry that could hide a vector
+            for (int it = 0; it < 4; ++it) {
+                solve(shift, v);
+                double s = 0.0;
+                for (double t : v) s += t * t;
+                for (double &t : v) t *= std::sqrt(0.5 / s);
+            }
+            out.push_back(v);
         }
-        return v;
+        return out;
     }
 
 private:
     int H;
     std::vector<double> d, o;
     double lo, hi;
-    // eigenvalues above x: positive pivots of A - x
-    int above(double x) const {
-        int n = 0;
-        double q = 1.0;
-        for (int u = 0; u < H; ++u) {
-            q = d[u] - x - (u ? o[u] * o[u] / q : 0.0);
-            if (q == 0.0) q = 1e-300;
-            n += q > 0.0;
-        }
-        return n;
-    }
     // v <- (A - x)^-1 v, Gaussian elimination with row exchanges (three diagonals above)
     void solve(double x, std::vector<double> &v) const {
         std::vector<double> a(H), b(H, 0.0), c(H, 0.0);   // the current upper rows: a b c at columns u, u+1, u+2
@@ -107,13 +116,18 @@ private:
     }
 };
 
+// About the rank band_basis finds at kBandTol for x = beta B degrees of freedom (x from 1 to 50).
+int rank_guess(double x) { return (int)std::ceil(x + 8.5 + 1.6 * std::log(std::max(1.0, x))); }
+
 // Basis [B/2][R] of the band |d| <= beta/2 (a row: R/2 even vectors, R/2 odd) of the least rank R that
 // the push kernels take whose residual over the band stays within tol; R = 0 if none does.  The residual
 // is the part of exp(-2 pi i d (u - c)) outside the basis, relative to its norm, checked on a grid of
 // d that holds the band's edge, where it is largest.
-std::vector<double> band_basis(int B, double beta, double tol, bool split, int *rank) {
+std::vector<double> band_basis(int B, double beta, double tol, int min_rank, int max_rank, int *rank) {
     const int H = B / 2, kD = 9;
     const Prolate even(B, beta, 0), odd(B, beta, 1);
+    const int most = std::min(max_rank, B - 4), guess = std::min(most, rank_guess(beta * B) + 4);
+    std::vector<std::vector<double>> ev = even.vectors(guess / 2 + 1), ov = odd.vectors(guess / 2 + 1);
     std::vector<std::vector<double>> vec, res(2 * kD, std::vector<double>(H));
     for (int i = 0; i < kD; ++i)
         for (int u = 0; u < H; ++u) {
@@ -122,10 +136,14 @@ std::vector<double> band_basis(int B, double beta, double tol, bool split, int *
             res[2 * i + 1][u] = std::sin(ph);
         }
     *rank = 0;
-    for (int R = 4; R == 4 || project_shape_ok(B, R, split); R += 4) {
+    for (int R = min_rank; R <= most; R += 4) {
+        if (R / 2 > (int)ev.size()) {
+            ev = even.vectors(most / 2);
+            ov = odd.vectors(most / 2);
+        }
         while ((int)vec.size() < R) {
             const int par = (int)vec.size() & 1;
-            vec.push_back((par ? odd : even).vector((int)vec.size() / 2));
+            vec.push_back((par ? ov : ev)[vec.size() / 2]);
             for (int i = 0; i < kD; ++i) {
                 std::vector<double> &r = res[2 * i + par];
                 double dot = 0.0;
@@ -133,7 +151,6 @@ std::vector<double> band_basis(int B, double beta, double tol, bool split, int *
                 for (int u = 0; u < H; ++u) r[u] -= dot * vec.back()[u];
             }
         }
-        if (R < 8) continue;
         double worst = 0.0;
         for (int i = 0; i < kD; ++i) {
             double e = 0.0;
@@ -156,15 +173,92 @@ std::vector<double> band_basis(int B, double beta, double tol, bool split, int *
 // of 2^-17 an element on the split path and FP32 sums of thousands of terms on the FP32 path.
 constexpr double kBandTol = 1e-7;
 
+}  // namespace
+
+namespace tacaw {
+const std::vector<double> &BandCache::basis(int B, double beta, int min_rank, int max_rank, int *rank) {
+    for (const Entry &e : entries)
+        if (e.B == B && e.beta == beta && e.max_rank == max_rank) {
+            *rank = e.rank;
+            return e.v;
+        }
+    Entry e{B, max_rank, 0, beta, {}};
+    e.v = band_basis(B, beta, kBandTol, min_rank, max_rank, &e.rank);
+    *rank = e.rank;
+    entries.push_back(std::move(e));
+    return entries.back().v;
+}
+}  // namespace tacaw
+
+namespace {
+
 // Segments and rings shorter than this keep staging frames: their passes are bound by launches.
 constexpr int kBandMinT = 512;
 
+// Two-level contraction of a form's coefficients (split path): superblock length S and rank r an energy
+// tile, for the least complex products a (row, frame): R / B of the first level's columns, r / S of the
+// energies, and 200 a coefficient written and read (16 bytes at the copy rate against 0.0128 ps a
+// product).  S = 0 where the direct sum over coefficients costs less than 1.18 times the best.  Measured
+// contractions, direct and two-level: 400 energies (work 208, 166) 6.3 and 4.1 ms on 2^20 rows x 2048
+// frames; 1000 energies (378, 222) 11.8 and 5.0 ms on 2^18 rows x 8192 frames.
+std::vector<double> choose_levels(const Stream &s, BandForm &b, std::vector<double> *centre, BandCache &cache) {
+    std::vector<double> best_w;
+    double width = 0.0;
+    const double dt = s.d.dt_fs * 1e-3 / kPlanck_meV_ps;
+    for (int g = 0; g < s.n_wt; ++g) {
+        const auto mm = std::minmax_element(s.E.begin() + (size_t)g * s.wt,
+                                            s.E.begin() + std::min((size_t)(g + 1) * s.wt, s.E.size()));
+        centre->push_back(0.5 * (*mm.first + *mm.second) * dt);
+        width = std::max(width, (*mm.second - *mm.first) * dt);
+    }
+    const int ring = std::min(s.ring, s.T);
+    const double best = (double)b.R / b.B * s.Nw_pad / 1.18;
+    // the better length by the estimated rank, then its basis
+    int best_S = 0;
+    auto cost_of = [&](int S, int r, int *wt1, int *n1) {
+        const int cols = s.n_wt * r;
+        *n1 = (cols + kDrainMaxOmegaTile - 1) / kDrainMaxOmegaTile;
+        *wt1 = (int)round_up((cols + *n1 - 1) / *n1, 16);
+        return (double)b.R / b.B * (*n1 * (*wt1 + 8)) + (double)r / S * s.Nw_pad + 200.0 * cols / S;
+    };
+    int wt1 = 0, n1 = 0;
+    double estimate = best;
+    for (int S : {256, 512}) {
+        if (S % b.B || S / b.B * b.R % 32 || S > ring || (s.needs_acc && s.ring % S)) continue;
+        const int r = rank_guess(width * S);
+        if (r > 56) continue;
+        const double c = cost_of(S, (int)round_up(r, 8), &wt1, &n1);
+        if (c < estimate) {
+            estimate = c;
+            best_S = S;
+        }
+    }
+    if (!best_S) return best_w;
+    const int S = best_S;
+    int r = 0;
+    const std::vector<double> &w = cache.basis(S, std::max(width, 1e-6), 4, 56, &r);
+    if (r == 0) return best_w;
+    // (the first level stores sectors of eight columns: other ranks are padded with zero vectors)
+    const int rp = (int)round_up(r, 8), z_slots = (int)round_up((int64_t)((ring + S - 1) / S) * rp, 32);
+    const double cost = cost_of(S, rp, &wt1, &n1);
+    if (cost >= best || b.z_begin() + s.n_wt * z_slots > s.ring) return best_w;
+    best_w.assign((size_t)(S / 2) * rp, 0.0);
+    for (int u = 0; u < S / 2; ++u)
+        for (int q = 0; q < r; ++q) best_w[(size_t)u * rp + (q < r / 2 ? q : q - r / 2 + rp / 2)] = w[(size_t)u * r + q];
+    b.work = cost;
+    b.S = S;
+    b.r = rp;
+    b.z_slots = z_slots;
+    b.wt1 = wt1;
+    b.n_wt1 = n1;
+    return best_w;
+}
 
 }  // namespace
 
 namespace tacaw {
 
-tacaw_status build_band_forms(tacaw_plan_s *p, Stream &s, int64_t room_bytes, cudaStream_t st) {
+tacaw_status build_band_forms(tacaw_plan_s *p, Stream &s, int64_t room_bytes, BandCache &cache, cudaStream_t st) {
     const bool split = p->prec == TACAW_PREC_SPLIT_BF16;
     if (p->in_place || (split && p->bf != 32) || s.T < kBandMinT) return TACAW_OK;
     const double dt_ps = s.d.dt_fs * 1e-3;
@@ -180,8 +274,8 @@ tacaw_status build_band_forms(tacaw_plan_s *p, Stream &s, int64_t room_bytes, cu
     for (int B : {32, 64, 128}) {
         if (!project_shape_ok(B, 8, split) || (s.needs_acc && s.ring % B)) continue;   // flushes end between blocks
         int R = 0;
-        const std::vector<double> basis = band_basis(B, std::max(beta, 1e-6), kBandTol, split, &R);
-        if (R == 0) continue;
+        const std::vector<double> &basis = cache.basis(B, std::max(beta, 1e-6), 8, 48, &R);
+        if (basis.empty() || !project_shape_ok(B, R, split)) continue;
         const int blocks = (std::min(s.ring, s.T) + B - 1) / B;
         BandForm b;
         b.B = B;
@@ -198,10 +292,17 @@ tacaw_status build_band_forms(tacaw_plan_s *p, Stream &s, int64_t room_bytes, cu
         ba.ring = s.ring;
         ba.slots = b.slots;
         ba.rounds = (s.T + s.ring - 1) / s.ring;
-        // one allocation: twiddles, responses (FP64), basis (FP64), modulation
-        const size_t rows = (size_t)ba.rounds * b.slots, n = basis.size(), tp = (size_t)round_up(s.T, B);
+        b.work = (double)R / B * s.Nw_pad;
+        std::vector<double> centre, w;
+        if (split) w = choose_levels(s, b, &centre, cache);
+        // one allocation: twiddles, first-level table, responses (FP64), basis (FP64), modulation, the second
+        // level's basis, group centres and each energy's
+        const int K = b.S ? b.r : R;
+        const size_t rows = (size_t)ba.rounds * (b.S ? b.z_slots : b.slots), n = basis.size();
+        const size_t tp = (size_t)round_up(s.T, B), n1 = (size_t)b.wt1 * b.n_wt1;
         const size_t tw = rows * s.Nw_pad * 8;   // bytes of B_hi, of B_lo, or of B32
-        const size_t bytes = (split ? 2 : 1) * tw + ((size_t)R * s.Nw + n + tp) * 8;
+        const size_t t1 = b.S ? (size_t)b.S / B * R * n1 * 8 : 0;   // of T_hi, of T_lo
+        const size_t bytes = (split ? 2 : 1) * tw + 2 * t1 + ((size_t)K * s.Nw + n + tp + w.size() + centre.size() + s.Nw) * 8;
         if ((int64_t)bytes > room_bytes) continue;
         unsigned char *mem = nullptr;
         if (!dev_alloc(p, &mem, bytes)) break;   // no memory for this form's tables: frames, or the form built before
@@ -211,18 +312,44 @@ tacaw_status build_band_forms(tacaw_plan_s *p, Stream &s, int64_t room_bytes, cu
             b.B_hi = reinterpret_cast<__nv_bfloat16 *>(q);
             b.B_lo = reinterpret_cast<__nv_bfloat16 *>(q + tw);
             q += 2 * tw;
+            b.T_hi = reinterpret_cast<__nv_bfloat16 *>(q);
+            b.T_lo = reinterpret_cast<__nv_bfloat16 *>(q + t1);
+            q += 2 * t1;
         } else {
             b.B32 = reinterpret_cast<float2 *>(q);
             q += tw;
         }
         double *d_resp = reinterpret_cast<double *>(q);
-        double *d_basis = d_resp + (size_t)R * s.Nw;
+        double *d_basis = d_resp + (size_t)K * s.Nw;
         b.mod = reinterpret_cast<float2 *>(d_basis + n);
+        double *d_w = reinterpret_cast<double *>(b.mod + tp), *d_centre = d_w + w.size(), *d_cj = d_centre + centre.size();
         b.basis.assign(basis.begin(), basis.end());
         CU_CHECK(p, cudaMemcpy(d_basis, basis.data(), sizeof(double) * n, cudaMemcpyHostToDevice), "basis");
         ba.basis = d_basis;
         const TableArgs ta = stream_table_args(s, p->bf);
         CU_CHECK(p, launch_band_mod(ta, ba, b.mod, st), "band modulation");
+        if (b.S) {
+            // first level, then the tiles' twiddles as those of blocks of S frames about each tile's centre
+            std::vector<double> cj(s.Nw);
+            for (int j = 0; j < s.Nw; ++j) cj[j] = centre[j / s.wt];
+            CU_CHECK(p, cudaMemcpy(d_w, w.data(), sizeof(double) * w.size(), cudaMemcpyHostToDevice), "basis");
+            CU_CHECK(p, cudaMemcpy(d_centre, centre.data(), sizeof(double) * centre.size(), cudaMemcpyHostToDevice), "centres");
+            CU_CHECK(p, cudaMemcpy(d_cj, cj.data(), sizeof(double) * s.Nw, cudaMemcpyHostToDevice), "centres");
+            BandMergeArgs ma{};
+            ma.b = ba;
+            ma.S = b.S;
+            ma.r = b.r;
+            ma.groups = s.n_wt;
+            ma.cols_pad = (int)n1;
+            ma.w = d_w;
+            ma.fg = d_centre;
+            CU_CHECK(p, launch_band_merge(ma, b.T_hi, b.T_lo, st), "band merge table");
+            ba.B = b.S;
+            ba.R = b.r;
+            ba.basis = d_w;
+            ba.fcj = d_cj;
+            ba.slots = b.z_slots;
+        }
         CU_CHECK(p, launch_band_response(ta, ba, d_resp, st), "band response");
         CU_CHECK(p, launch_band_twiddles(ta, ba, d_resp, b.B_hi, b.B_lo, b.B32, st), "band twiddles");
         s.band[s.n_band++] = b;
@@ -234,12 +361,12 @@ tacaw_status build_band_forms(tacaw_plan_s *p, Stream &s, int64_t room_bytes, cu
 // frames a push; 60 to 1000 energies): a push of frames 2.7 + 24 / n (5.7 where n is no multiple of 4 and
 // takes the unaligned conversion); a push of whole blocks 2.2 + 36 / n, and where it ends inside blocks
 // 3.2 for the share of the frames that pass through the carry and 16 / n for the extra launch's rows; the
-// contraction 0.0128 (split) or 0.142 (FP32) an energy, times 1.25 or 1.12 R / B on coefficients (shorter
+// contraction 0.0128 (split) or 0.142 (FP32) a product, 1.25 or 1.12 times that on coefficients (shorter
 // sums under the same epilogue).
 int choose_form(const tacaw_plan_s *p, const Stream &s, int n) {
     const bool split = p->prec == TACAW_PREC_SPLIT_BF16;
-    const double energies = (split ? 0.0128 : 0.142) * s.Nw_pad, stretch = split ? 1.25 : 1.12;
-    double best = 0.97 * ((n % 4 == 0 || !split ? 2.7 + 24.0 / n : 5.7) + energies);
+    const double product = split ? 0.0128 : 0.142, stretch = split ? 1.25 : 1.12;
+    double best = 0.97 * ((n % 4 == 0 || !split ? 2.7 + 24.0 / n : 5.7) + product * s.Nw_pad);
     int form = -1;
     for (int i = 0; i < s.n_band; ++i) {
         const BandForm &b = s.band[i];
@@ -248,7 +375,7 @@ int choose_form(const tacaw_plan_s *p, const Stream &s, int n) {
         // below a block (they drift against the blocks), a block's worth for longer ones
         const double f = n % b.B == 0 ? 0.0 : b.B % n == 0 ? 1.0 - (double)n / b.B : n < b.B ? 1.0 : (double)b.B / n;
         const double push = 2.2 + 36.0 / std::max(n, 32) + (f > 0.0 ? 3.2 * f + 16.0 / n : 0.0);
-        const double cost = push + stretch * b.R / b.B * energies;
+        const double cost = push + stretch * product * b.work;
         if (cost < best) {
             best = cost;
             form = i;

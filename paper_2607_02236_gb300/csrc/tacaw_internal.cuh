@@ -284,6 +284,7 @@ struct BandTableArgs {
     int B, R;
     double fc;
     const double *basis;
+    const double *fcj;         // [Nw] band centre of each energy's group (null: fc)
     int ring;                  // frames per flush (a multiple of B, or >= T)
     int slots;                 // table rows per flush (whole K-blocks of 32 on the split path)
     int rounds;                // flushes a segment
@@ -294,6 +295,16 @@ cudaError_t launch_band_response(const TableArgs &t, const BandTableArgs &b, dou
 // split twiddles [rounds * slots / 32][2 Nw_pad][64] (pre-swizzled) or FP32 [rounds * slots][Nw_pad]
 cudaError_t launch_band_twiddles(const TableArgs &t, const BandTableArgs &b, const double *q_resp,
                                  __nv_bfloat16 *B_hi, __nv_bfloat16 *B_lo, float2 *B32, cudaStream_t st);
+
+// First-level table of the two-level contraction (fp16 hi/lo, pre-swizzled, [S R / B / 32][2 cols_pad][64]):
+// coefficients of a superblock of S frames (S / B blocks on b's basis) -> r coefficients of each energy
+// group g on the basis w ([S/2][r] rows of its first half, FP64) shifted to the group's centre fg[g].
+struct BandMergeArgs {
+    BandTableArgs b;
+    int S, r, groups, cols_pad;
+    const double *w, *fg;
+};
+cudaError_t launch_band_merge(const BandMergeArgs &m, __nv_bfloat16 *T_hi, __nv_bfloat16 *T_lo, cudaStream_t st);
 
 cudaError_t launch_mean(const FrameGeom &g, int n, float2 *mu_hat, cudaStream_t st);
 // f16 != 0: fp16 hi/lo pieces of f16_scale * (psi - mu_hat); a scaled component beyond the
@@ -376,6 +387,16 @@ struct TcPlanArgs {
     int f16;                   // operands are fp16 pieces (split-FP16 path, band-limited staging) instead of bf16
     const float *row_scale;    // band-limited staging: [M_pad] power of two the row's coefficients are scaled by
     float row_unit;            // (0: an empty row); its sums times row_unit / row_scale are the flush's result
+    // Two-level band-limited contraction.  First level (z_hi set): n_sb superblocks of n_kb staging blocks
+    // each (total_kb in all), every one with the same table, a tile per (row tile, superblock, column
+    // tile); column c of superblock b is coefficient c mod z_r of energy group c / z_r, stored times z_mul as
+    // fp16 hi + lo at slot b z_r + c mod z_r of the group's staged rows [z_slots / 32][M_pad][64].
+    // Second level: energy tile w reads the staged rows of group w, a_group bytes apart.
+    int n_sb, total_kb;
+    void *z_hi, *z_lo;
+    int z_r, z_cols, z_slots;
+    float z_mul;
+    int64_t a_group;
     unsigned long long *trace; // null, or kTraceWords globaltimer stamps per CTA (phase boundaries)
     uint32_t *err;
     uint64_t wait_ns;          // pipeline waits give up after this many ns (0: the default 4 s)

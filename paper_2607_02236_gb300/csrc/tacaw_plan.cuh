@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
 
+#include <list>
 #include <string>
 #include <utility>
 #include <vector>
@@ -19,12 +20,25 @@ namespace tacaw {
 struct BandForm {
     int B = 0, R = 0;
     double beta = 0.0;         // the band's width (with B and R: the basis)
+    double work = 0.0;         // complex products a (row, frame) of the contraction (choose_levels)
     int slots = 0;             // table rows per flush; the carry, then the row scales, follow
                                // the ring's first `slots` slots
     float2 *mod = nullptr;     // [T rounded up to B]
     std::vector<float> basis;  // [B/2][R]
     __nv_bfloat16 *B_hi = nullptr, *B_lo = nullptr;   // twiddles (split path)
     float2 *B32 = nullptr;                            // twiddles (FP32 path)
+    // two-level contraction (split path, S > 0): superblocks of S frames first become r coefficients per
+    // energy tile (T_hi, T_lo), staged behind the row scales; B_hi, B_lo then are the tiles' twiddles over
+    // z_slots of those
+    int S = 0, r = 0, z_slots = 0;
+    int wt1 = 0, n_wt1 = 0;    // column tiles of the first level (n_wt groups of r columns)
+    __nv_bfloat16 *T_hi = nullptr, *T_lo = nullptr;
+    int z_begin() const { return (slots + 2 * B + 1 + 31) / 32 * 32; }   // first staging slot of theirs
+    int z_shift() const {      // their scale is 2^-z_shift of the row's: sqrt(2 S R / B) 2^15 stays below 65504
+        int k = 0;
+        while ((double)(1 << k) * 1.99 < __builtin_sqrt(2.0 * S * R / B)) ++k;
+        return k;
+    }
 };
 constexpr int kBandForms = 2;
 constexpr int kBandDrainBlocks = 10;   // staging blocks per drained H chunk on band-limited forms
@@ -206,9 +220,19 @@ tacaw_status check_plan(tacaw_plan_s *p);
 tacaw_status check_kernel_memory(const void *ptr, const char *what, bool allow_host, cudaStream_t st);
 // Waits for `st` and turns the device error word into a status (poisoning the plan).
 tacaw_status read_device_error(tacaw_plan_s *p, cudaStream_t st);
+// Bases computed during one plan creation (the streams of a plan mostly share their bands).
+struct BandCache {
+    struct Entry {
+        int B, max_rank, rank;
+        double beta;
+        std::vector<double> v;
+    };
+    std::list<Entry> entries;
+    const std::vector<double> &basis(int B, double beta, int min_rank, int max_rank, int *rank);
+};
 // Builds the band-limited staging forms that pay for stream s (tacaw_band.cu), within room_bytes of
 // device memory; a stream without any keeps staging frames.
-tacaw_status build_band_forms(tacaw_plan_s *p, Stream &s, int64_t room_bytes, cudaStream_t st);
+tacaw_status build_band_forms(tacaw_plan_s *p, Stream &s, int64_t room_bytes, BandCache &cache, cudaStream_t st);
 // The staging form a ring takes whose first push has n frames (-1: frames).
 int choose_form(const tacaw_plan_s *p, const Stream &s, int n);
 // Table arguments of stream s after its tables were built.

@@ -42,7 +42,10 @@ CASES = [(513, 200, 120.0, [32], 0),           # a last block of one frame
          (700, 260, 60.0, [20], 0),            # every block through the carry
          (1024, 300, 120.0, [32], 256),        # four flushes
          (1152, 500, 150.0, [128, 256], 384),  # three flushes, pushes across ring ends
-         (2048, 130, 120.0, [8, 24], 0)]
+         (2048, 130, 120.0, [8, 24], 0),
+         # two-level sums: nine energy tiles, a last superblock of 33 frames, rings of two superblocks
+         (2081, 950, 150.0, [64], 0),
+         (4096, 1000, 150.0, [64, 128], 1024)]
 
 
 @pytest.mark.parametrize("precision", ["split_bf16", "fp32"])
