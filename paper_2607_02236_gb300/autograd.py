@@ -17,6 +17,12 @@ def _dims(plan: TacawPlan, sid: int):
     return s, nw, len(s.detectors)
 
 
+def _total_frames(s):
+    """Frames of a stream's whole push sequence."""
+    n_seg = max(1, int(s.welch_segments))
+    return int(s.skip_init) + (n_seg - 1) * (int(s.welch_stride) or s.T) + s.T
+
+
 class TacawSpectrum(torch.autograd.Function):
     """S = TacawSpectrum.apply(frames, plan, stream_id, frames_per_push).
 
@@ -33,8 +39,7 @@ class TacawSpectrum(torch.autograd.Function):
         s, nw, D = _dims(plan, stream_id)
         cs = torch.cuda.current_stream()
         plan.reset(cs)
-        n_seg = max(1, int(s.welch_segments))
-        total = int(s.skip_init) + (n_seg - 1) * (int(s.welch_stride) or s.T) + s.T
+        total = _total_frames(s)
         chunk = frames_per_push or total
         base = frames.data_ptr()
         for t0 in range(0, total, chunk):
@@ -51,7 +56,13 @@ class TacawSpectrum(torch.autograd.Function):
     @staticmethod
     def backward(ctx, gS):
         (frames,) = ctx.saved_tensors
-        grad = torch.zeros_like(frames)
+        # tacaw_backward writes every ROI element: only frames larger than the ROI need the zeros beside it
+        s = ctx.plan.streams[ctx.sid]
+        roi_only = (s.roi_x0 == 0 and s.roi_y0 == 0 and s.pitch_row == s.kx
+                    and (s.n_probes == 1 or s.pitch_probe == s.kx * s.ky)
+                    and s.pitch_frame == s.n_probes * s.kx * s.ky and frames.is_contiguous()
+                    and frames.numel() == _total_frames(s) * s.pitch_frame)
+        grad = torch.empty_like(frames) if roi_only else torch.zeros_like(frames)
         ctx.plan.backward(ctx.sid, gS.contiguous().to(torch.float32), frames, grad, torch.cuda.current_stream())
         return grad, None, None, None
 

@@ -16,7 +16,21 @@ __global__ void aperture_kernel(ApertureArgs a) {
     if (j >= a.Nw) return;
     const float *Ipj = a.I + ((int64_t)p * a.Nw + j) * a.npix;
     float v = 0.f;
-    for (int i = a.off[d] + lane; i < a.off[d + 1]; i += 32) v = fmaf(a.wts[i], Ipj[a.idx[i]], v);
+    // eight pixels in flight a lane, added in list order (one at a time the list of a 20-pixel disk, 40
+    // dependent pairs of loads, took 15 us)
+    const int end = a.off[d + 1];
+    for (int i0 = a.off[d] + lane; i0 < end; i0 += 256) {
+        float x[8], w[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const int i = i0 + 32 * k;
+            w[k] = i < end ? a.wts[i] : 0.f;
+            x[k] = i < end ? Ipj[a.idx[i]] : 0.f;
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+            if (i0 + 32 * k < end) v = fmaf(w[k], x[k], v);
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     if (lane == 0) a.S[((int64_t)p * a.D + d) * a.Nw + j] = v;

@@ -13,11 +13,10 @@
 namespace tacaw {
 
 __device__ __forceinline__ const float2 *row_src(const FrameGeom &g, int64_t m) {
-    int64_t p = m / g.npix;
-    int64_t pix = m - p * g.npix;
-    int64_t y = pix / g.kx;
-    int64_t x = pix - y * g.kx;
-    return g.base + p * g.pitch_probe + (g.roi_y0 + y) * g.pitch_row + (g.roi_x0 + x);
+    // (rows fit 32 bits, checked at plan creation: 64-bit divisions are several times as long)
+    const uint32_t p = (uint32_t)m / (uint32_t)g.npix, pix = (uint32_t)m - p * (uint32_t)g.npix;
+    const uint32_t y = pix / (uint32_t)g.kx, x = pix - y * (uint32_t)g.kx;
+    return g.base + (int64_t)p * g.pitch_probe + (int64_t)(g.roi_y0 + (int)y) * g.pitch_row + (g.roi_x0 + (int)x);
 }
 
 // Provisional mean of each row over the first n frames of the first push (launch_mean caps n).  Block = 32 rows x 8
@@ -104,7 +103,7 @@ __host__ __device__ __forceinline__ int swz_word(int w, int64_t m, int bf, int s
     return ((((w >> 2) ^ sw)) << 2) | (w & 3);
 }
 
-// Staged frame slot s (s0 + t) goes to block s/bf, elements 2(s%bf), 2(s%bf)+1 of row m
+// Blocks of 8 frames.  Staged frame slot s (s0 + t) goes to block s/bf, elements 2(s%bf), 2(s%bf)+1 of row m
 // (rows of 2*bf bf16 = 4*bf bytes; bf is 8, 16 or 32).
 template <bool F16>
 __global__ void convert_split_kernel(FrameGeom g, int n, int s0, int bf, int64_t M_pad, const float2 *mu_hat,
@@ -177,17 +176,20 @@ __global__ void convert_split_kernel(FrameGeom g, int n, int s0, int bf, int64_t
     if (F16 && amax > kF16Max) atomicOr(err, DEVERR_FP16_RANGE);
 }
 
-// Staging blocks of BF frames, 128 rows per CTA, for pushes whose start s0 and length n are
-// multiples of 4 frames (one 16-byte chunk of a row): the push is walked in pieces that each
+// Staging blocks of BF frames, 128 rows per CTA: the push is walked in pieces that each
 // lie inside one block (a whole block, or part of one when a push is shorter than a block or
-// starts inside one).  Each thread converts its row's frames of the piece into a shared tile
+// starts inside one).  A piece that starts or ends inside a 16-byte chunk (4 frames) writes that
+// chunk's words alone; a whole push of such pieces (25 frames of 8 235 rows) took 12.3 us a push in the
+// word-by-word kernel that now serves 8-frame blocks only.  Each thread converts its row's frames of the piece into a shared tile
 // (16-byte chunks XOR-swizzled by row to spread the banks); the CTA then writes the piece's
 // chunks of the 128 rows with consecutive threads on consecutive chunks.  The stored swizzle
 // only exchanges chunks inside 32-byte sectors, so a piece always writes whole sectors.
 // The rows of block `blk` (rows 128 blk ..) of one push; run by 128 threads.  PF: the longest
 // piece the caller passes (BF, or 16 for pushes of at most 16 frames: half the registers and
 // shared memory, twice the CTAs an SM holds; the pieces, and so the sums, are the same).
-template <int BF, int PF, bool F16>
+// ALIGNED: start and length are multiples of 4 frames (no partial chunks; their handling made a 64-frame push
+// of 1 682 rows 10.3 us instead of 8.3).
+template <int BF, int PF, bool F16, bool ALIGNED>
 __device__ __forceinline__ void convert_tiled_rows(const FrameGeom &g, int n, int s0, int64_t M_pad,
                                                    const float2 *mu_hat, double2 *sum_res, __nv_bfloat16 *A_hi,
                                                    __nv_bfloat16 *A_lo, int swz, float sc, uint32_t *err, int64_t blk) {
@@ -207,12 +209,14 @@ __device__ __forceinline__ void convert_tiled_rows(const FrameGeom &g, int n, in
     float amax = 0.f;
     for (int t0 = 0; t0 < n;) {
         const int f0 = (s0 + t0) % bf;                 // first frame of the piece inside its block
-        const int len = min(bf - f0, n - t0);          // a multiple of 4
-        const int c0 = f0 / 4, nc = len / 4;
-        float2 v[PF];
+        const int lead = ALIGNED ? 0 : f0 & 3;         // words of its first chunk before it
+        const int len = min(min(bf - f0, n - t0), PF - lead);
+        const int c0 = f0 / 4, end = lead + len, nc = (end + 3) / 4;
+        float2 v[PF];                                  // by word of the piece's chunks; others stay at the mean
 #pragma unroll
         for (int i = 0; i < PF; ++i)
-            v[i] = (valid && i < len) ? __ldcs(src + (int64_t)(t0 + i) * g.pitch_frame) : make_float2(0.f, 0.f);
+            v[i] = (valid && i >= lead && i < end) ? __ldcs(src + (int64_t)(t0 + i - lead) * g.pitch_frame)
+                                                   : (ALIGNED ? make_float2(0.f, 0.f) : mu);
         float br = 0.f, bi = 0.f;
 #pragma unroll
         for (int k = 0; k < lcpr; ++k) {
@@ -238,8 +242,16 @@ __device__ __forceinline__ void convert_tiled_rows(const FrameGeom &g, int n, in
             const int slot = rr * lcpr + (k ^ (rr & (lcpr - 1)));
             // stored chunk position of chunk c (m0 is a multiple of 128: row rr's pattern)
             const int cs = swz ? (c ^ (((rr * cpr) >> 3) & (cpr - 1))) : c;
-            Hi[base + rr * cpr + cs] = tile_h[slot];
-            Lo[base + rr * cpr + cs] = tile_l[slot];
+            const int w0 = max(lead - 4 * k, 0), w1 = min(end - 4 * k, 4);
+            if (ALIGNED || w1 - w0 == 4) {
+                Hi[base + rr * cpr + cs] = tile_h[slot];
+                Lo[base + rr * cpr + cs] = tile_l[slot];
+            } else {
+                for (int w = w0; w < w1; ++w) {
+                    reinterpret_cast<uint32_t *>(Hi + base + rr * cpr + cs)[w] = reinterpret_cast<uint32_t *>(tile_h + slot)[w];
+                    reinterpret_cast<uint32_t *>(Lo + base + rr * cpr + cs)[w] = reinterpret_cast<uint32_t *>(tile_l + slot)[w];
+                }
+            }
         }
         __syncthreads();
         t0 += len;
@@ -253,12 +265,12 @@ __device__ __forceinline__ void convert_tiled_rows(const FrameGeom &g, int n, in
     if (F16 && amax > kF16Max) atomicOr(err, DEVERR_FP16_RANGE);
 }
 
-template <int BF, int PF, bool F16>
+template <int BF, int PF, bool F16, bool ALIGNED>
 __global__ void __launch_bounds__(128) convert_split_tiled_kernel(FrameGeom g, int n, int s0, int64_t M_pad,
                                                                   const float2 *mu_hat, double2 *sum_res,
                                                                   __nv_bfloat16 *A_hi, __nv_bfloat16 *A_lo, int swz,
                                                                   float sc, uint32_t *err) {
-    convert_tiled_rows<BF, PF, F16>(g, n, s0, M_pad, mu_hat, sum_res, A_hi, A_lo, swz, sc, err, blockIdx.x);
+    convert_tiled_rows<BF, PF, F16, ALIGNED>(g, n, s0, M_pad, mu_hat, sum_res, A_hi, A_lo, swz, sc, err, blockIdx.x);
 }
 
 // One push of each of several streams in one launch: CTA b converts block b - e.cta_begin of
@@ -269,10 +281,11 @@ __global__ void __launch_bounds__(128) convert_split_group_kernel(const __grid_c
     int k = 0;
     while (k + 1 < cg.n && (int64_t)blockIdx.x >= cg.e[k + 1].cta_begin) ++k;
     const ConvEntry &e = cg.e[k];
-    convert_tiled_rows<BF, PF, F16>(e.g, e.n, e.s0, e.M_pad, e.mu_hat, e.sum_res, e.A_hi, e.A_lo, swz, sc, err,
+    convert_tiled_rows<BF, PF, F16, true>(e.g, e.n, e.s0, e.M_pad, e.mu_hat, e.sum_res, e.A_hi, e.A_lo, swz, sc, err,
                                     (int64_t)blockIdx.x - e.cta_begin);
 }
 
+// FP32 staging, one thread a row.
 __global__ void convert_fp32_kernel(FrameGeom g, int n, int s0, int64_t M_pad, const float2 *mu_hat,
                                     double2 *sum_res, float2 *A32) {
     int64_t m = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -307,6 +320,47 @@ __global__ void convert_fp32_kernel(FrameGeom g, int n, int s0, int64_t M_pad, c
     a.x += sr;
     a.y += si;
     sum_res[m] = a;
+}
+
+// The same for long pushes of few rows.  Block = 32 rows x 8 frame lanes, as in mean_kernel: lane f takes frames f, f + 8, ..., eight
+// of them in flight, and the eight FP64 partial sums of a row are added in a fixed order.  (One thread a
+// row took 30 us for one push of 256 frames of 2^14 rows: a chain of 32 batches of loads.)
+__global__ void __launch_bounds__(256) convert_fp32_lanes_kernel(FrameGeom g, int n, int s0, int64_t M_pad,
+                                                                 const float2 *mu_hat, double2 *sum_res, float2 *A32) {
+    __shared__ double2 part[8][32];
+    const int r = threadIdx.x & 31, f = threadIdx.x >> 5;
+    const int64_t m = (int64_t)blockIdx.x * 32 + r;
+    const bool valid = m < g.M;
+    const float2 *src = valid ? row_src(g, m) : nullptr;
+    const float2 mu = valid ? mu_hat[m] : make_float2(0.f, 0.f);
+    double sr = 0.0, si = 0.0;
+    for (int t0 = f; t0 < n; t0 += 64) {
+        float2 v[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            v[i] = valid && t0 + 8 * i < n ? __ldcs(src + (int64_t)(t0 + 8 * i) * g.pitch_frame) : mu;
+        float br = 0.f, bi = 0.f;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const float2 q = make_float2(v[i].x - mu.x, v[i].y - mu.y);
+            br += q.x;
+            bi += q.y;
+            if (valid && t0 + 8 * i < n) A32[(size_t)(s0 + t0 + 8 * i) * M_pad + m] = q;
+        }
+        sr += br;
+        si += bi;
+    }
+    part[f][r] = make_double2(sr, si);
+    __syncthreads();
+    if (f == 0 && valid) {
+        double2 a = sum_res[m];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            a.x += part[k][r].x;
+            a.y += part[k][r].y;
+        }
+        sum_res[m] = a;
+    }
 }
 
 // Zeroes staged slots [staged, next multiple of bf) of the last block, all M_pad rows.
@@ -354,17 +408,18 @@ template <bool F16>
 static cudaError_t convert_split(const FrameGeom &g, int n, int s0, int bf, int64_t M_pad, const float2 *mu_hat,
                                  double2 *sum_res, __nv_bfloat16 *A_hi, __nv_bfloat16 *A_lo, int swz, float sc,
                                  uint32_t *err, cudaStream_t st) {
-    if (convert_split_groupable(bf, s0, n)) {
+    if (bf >= 16) {
         const unsigned grid = (unsigned)(M_pad / 128);
+        const bool aligned = convert_split_groupable(bf, s0, n);
+        void (*kern)(FrameGeom, int, int, int64_t, const float2 *, double2 *, __nv_bfloat16 *, __nv_bfloat16 *, int,
+                     float, uint32_t *);
         if (bf == 32 && n > 16)
-            convert_split_tiled_kernel<32, 32, F16><<<grid, 128, 0, st>>>(g, n, s0, M_pad, mu_hat, sum_res, A_hi,
-                                                                          A_lo, swz, sc, err);
+            kern = aligned ? convert_split_tiled_kernel<32, 32, F16, true> : convert_split_tiled_kernel<32, 32, F16, false>;
         else if (bf == 32)
-            convert_split_tiled_kernel<32, 16, F16><<<grid, 128, 0, st>>>(g, n, s0, M_pad, mu_hat, sum_res, A_hi,
-                                                                          A_lo, swz, sc, err);
+            kern = aligned ? convert_split_tiled_kernel<32, 16, F16, true> : convert_split_tiled_kernel<32, 16, F16, false>;
         else
-            convert_split_tiled_kernel<16, 16, F16><<<grid, 128, 0, st>>>(g, n, s0, M_pad, mu_hat, sum_res, A_hi,
-                                                                          A_lo, swz, sc, err);
+            kern = aligned ? convert_split_tiled_kernel<16, 16, F16, true> : convert_split_tiled_kernel<16, 16, F16, false>;
+        kern<<<grid, 128, 0, st>>>(g, n, s0, M_pad, mu_hat, sum_res, A_hi, A_lo, swz, sc, err);
         return cudaGetLastError();
     }
     convert_split_kernel<F16><<<blocks_for(g.M, 256), 256, 0, st>>>(g, n, s0, bf, M_pad, mu_hat, sum_res, A_hi,
@@ -412,7 +467,12 @@ cudaError_t launch_convert_split_group(ConvGroup &cg, int bf, int swz, int f16, 
 
 cudaError_t launch_convert_fp32(const FrameGeom &g, int n, int s0, int64_t M_pad, const float2 *mu_hat,
                                 double2 *sum_res, float2 *A32, cudaStream_t st) {
-    convert_fp32_kernel<<<blocks_for(g.M, 256), 256, 0, st>>>(g, n, s0, M_pad, mu_hat, sum_res, A32);
+    // frame lanes where the push gives each several frames and one thread a row would leave SMs short of
+    // warps (8-frame pushes of 2^17 rows took half as long again with lanes: their FP64 sums and divisions)
+    if (n >= 64 && g.M <= (int64_t)1 << 16)
+        convert_fp32_lanes_kernel<<<blocks_for(g.M, 32), 256, 0, st>>>(g, n, s0, M_pad, mu_hat, sum_res, A32);
+    else
+        convert_fp32_kernel<<<blocks_for(g.M, 256), 256, 0, st>>>(g, n, s0, M_pad, mu_hat, sum_res, A32);
     return cudaGetLastError();
 }
 
