@@ -357,16 +357,17 @@ tacaw_status build_band_forms(tacaw_plan_s *p, Stream &s, int64_t room_bytes, Ba
     return TACAW_OK;
 }
 
-// The form with the least time a (row, frame), from measurements in picoseconds on 2^18 rows (16 to 64
-// frames a push; 60 to 1000 energies): a push of frames 2.7 + 24 / n (5.7 where n is no multiple of 4 and
-// takes the unaligned conversion); a push of whole blocks 2.2 + 36 / n, and where it ends inside blocks
-// 3.2 for the share of the frames that pass through the carry and 16 / n for the extra launch's rows; the
-// contraction 0.0128 (split) or 0.142 (FP32) a product, 1.25 or 1.12 times that on coefficients (shorter
-// sums under the same epilogue).
+// The form with the least time a (row, frame), in picoseconds, fitted to measurements (2^16 to 2^20 rows, 8 to
+// 64 frames a push, 60 to 1000 energies): a push of frames 2.65 + 8 / n and 3 us a launch (0.5 more where it
+// parts the 16-byte chunks of 4 frames); a push of whole blocks 2.3 + 8 / n and 4 us a launch, and 3.7 for
+// the share of the frames that passes through the carry; the contraction 0.0139 (split) or 0.142 (FP32) a
+// product, a tenth more on coefficients (shorter sums, drained more often).  Both sides at the line: six
+// partitions pushed 16 frames at a time, 300 energies: frames 14.9 + 20.1 ms, blocks of 32 with
+// half their frames carried 21.2 + 11.0 ms.
 int choose_form(const tacaw_plan_s *p, const Stream &s, int n) {
     const bool split = p->prec == TACAW_PREC_SPLIT_BF16;
-    const double product = split ? 0.0128 : 0.142, stretch = split ? 1.25 : 1.12;
-    double best = 0.97 * ((n % 4 == 0 || !split ? 2.7 + 24.0 / n : 5.7) + product * s.Nw_pad);
+    const double product = split ? 0.0139 : 0.142, push_rows = (double)s.M * n;
+    double best = 0.97 * (2.65 + 8.0 / n + 3e6 / push_rows + (n % 4 ? 0.5 : 0.0) + product * s.Nw_pad);
     int form = -1;
     for (int i = 0; i < s.n_band; ++i) {
         const BandForm &b = s.band[i];
@@ -374,8 +375,7 @@ int choose_form(const tacaw_plan_s *p, const Stream &s, int n) {
         // none for whole blocks, all but the completing push's for parts of a block, all for other sizes
         // below a block (they drift against the blocks), a block's worth for longer ones
         const double f = n % b.B == 0 ? 0.0 : b.B % n == 0 ? 1.0 - (double)n / b.B : n < b.B ? 1.0 : (double)b.B / n;
-        const double push = 2.2 + 36.0 / std::max(n, 32) + (f > 0.0 ? 3.2 * f + 16.0 / n : 0.0);
-        const double cost = push + stretch * product * b.work;
+        const double cost = 2.3 + 8.0 / std::max(n, 32) + 4e6 / push_rows + 3.7 * f + 1.1 * product * b.work;
         if (cost < best) {
             best = cost;
             form = i;
