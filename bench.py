@@ -228,6 +228,20 @@ def ffma_roofline(cmac_launch, kernel_ms, kname, launches_per_step, sm_max_mhz):
             "peak_source": "152 SMs x 128 FP32 lanes x 2 flop x max SM clock"}
 
 
+def step_roofline(bytes_step, ms_step, kernel_ms, kname, launches_per_step):
+    """HBM roofline of a whole step: the bytes it cannot do without (the ROI of every frame read once,
+    the intensities written once) over the step's time, against the measured copy bandwidth.  Band-limited
+    staging and the two-level contraction do a fraction of the products `value` counts (rows x T x
+    energies of the transform), so no fixed flop count per counted product describes the contraction."""
+    peaks, src = measured_peaks()
+    hbm = peaks.get("hbm_gbs")
+    ach = bytes_step / (ms_step * 1e-3) / 1e9
+    return {"bound": "hbm", "achieved": ach, "peak": hbm, "unit": "GB/s", "frac": ach / hbm if hbm else None,
+            "traffic": None, "kernel": kname, "kernel_ms": kernel_ms, "launches_per_step": launches_per_step,
+            "bytes_per_step": bytes_step, "ms_per_step": ms_step,
+            "peak_source": f"{src} copy bandwidth (MEASURED_PEAKS.json hbm_gbs)"}
+
+
 def step_spread(per_step):
     """Median, min and max of the timed steps' own durations (ms)."""
     if not per_step:
@@ -236,13 +250,13 @@ def step_spread(per_step):
 
 
 def conversion_roofline(bytes_per_step, ms_per_step, split=True):
-    """HBM roofline of the pushes: each conversion reads a complex64 sample (8 B) and writes its two
-    16-bit pieces of Re and Im (or a float2 on the FP32 path): 16 B per (row, frame)."""
+    """HBM roofline of the pushes by what they cannot do without: each complex64 sample (8 B) read once.
+    What they write depends on the staging form (8 B a sample as frames, 8 R / B as block coefficients)."""
     peaks, src = measured_peaks()
     hbm = peaks.get("hbm_gbs")
     ach = bytes_per_step / (ms_per_step * 1e-3) / 1e9
     return {"bound": "hbm", "achieved": ach, "peak": hbm, "unit": "GB/s", "frac": ach / hbm if hbm else None,
-            "traffic": None, "kernel": "convert_split_tiled_kernel" if split else "convert_fp32_kernel",
+            "traffic": None, "kernel": "project_group_kernel / " + ("convert_split_tiled_kernel" if split else "convert_fp32_kernel"),
             "bytes_per_step": bytes_per_step, "ms_per_step": ms_per_step,
             "timed": "CUDA events around reset + all pushes of each batch or segment (the span also holds the "
                      "provisional-mean kernel of the first push, whose reads are not counted)",
@@ -550,9 +564,8 @@ def thick_leg(ctx, args):
         err = max(err, e)
         cpu = cb or cpu
 
-    roof = tensor_roofline(cmac_step / max(k_per_step, 1), flush_ms, "flush_tc_drain2_kernel", k_per_step,
-                           workload="thick")
-    conv = conversion_roofline(16.0 * B * npix * T * n_batch, push_ms)
+    roof = step_roofline(n_batch * B * npix * (8.0 * T + 4.0 * Nw), ms, flush_ms, "flush_tc_drain2_kernel", k_per_step)
+    conv = conversion_roofline(8.0 * B * npix * T * n_batch, push_ms)
 
     # end to end through the public API from pinned host memory: the same step with the ring in
     # host memory -- the push kernels read each push's ROI rows over the host link (zero-copy
@@ -619,8 +632,12 @@ def thick_leg(ctx, args):
                        "full_grid": f"{gx}x{gy}", "k_roi": f"{K}x{K} at ({rx}, {ry})", "T": T,
                        "frames_per_push": Tc, "n_omega": Nw, "E_range_meV": [0, spec.E_max_meV],
                        "window": spec.window, "detectors": D,
-                       "precision": "split_bf16: hi*hi + hi*lo + lo*hi, fp32 accumulate in tensor memory, hi*hi "
-                                    f"drained into fp32 registers every {info['tc_drain_frames']} frames, fp64 phase",
+                       "precision": "split_bf16 plan: hi*hi + hi*lo + lo*hi, fp32 accumulate in tensor memory, hi*hi "
+                                    "drained into fp32 registers (frames every "
+                                    f"{info['tc_drain_frames']}, block coefficients every 128 to 320 slots), fp64 "
+                                    "phase; 64-frame blocks staged as fp16 hi + lo coefficients on the energies' band",
+                       "value_counts": "rows x T x energies of the transform per step; band-limited staging and the "
+                                       "two-level contraction reach the same result in fewer products",
                        "k_stage": info["k_stage"], "flushes_per_batch": -(-T // info["k_stage"]),
                        "accumulators": ["kahan", "fp64", "fp32"][info["accum"]] if info["k_stage"] < T else "none",
                        "omega_tile": info["omega_tile"], "tc_block_frames": info["tc_block_frames"],
@@ -770,13 +787,14 @@ def realistic_leg(ctx, args, sample_clocks=True):
     err = error()
     phases = flush_phases(plan, lambda k: run(plan)) if args.trace and split else None
     plan.close()
-    if split:
-        kname = "flush_tc_inplace_kernel" if info["frames_in_place"] else "flush_tc_drain2_kernel"
-        roof = tensor_roofline(cmac_step / max(k_per_step, 1), flush_ms, kname, k_per_step, args.precision)
+    bytes_step = P * npix * (8.0 * T + 4.0 * Nw)
+    if info["frames_in_place"]:
+        roof = tensor_roofline(cmac_step / max(k_per_step, 1), flush_ms, "flush_tc_inplace_kernel", k_per_step,
+                               args.precision)
     else:
-        roof = ffma_roofline(cmac_step / max(k_per_step, 1), flush_ms, "flush_simt_kernel", k_per_step,
-                             (clocks or {}).get("sm_max_mhz"))
-    conv = None if info["frames_in_place"] else conversion_roofline(16.0 * P * npix * T, push_ms, split)
+        roof = step_roofline(bytes_step, ms, flush_ms, "flush_tc_drain2_kernel" if split else "flush_simt_kernel",
+                             k_per_step)
+    conv = None if info["frames_in_place"] else conversion_roofline(8.0 * P * npix * T, push_ms, split)
 
     def comparison(precision, steps):
         with TacawPlan([stream_config(spec)], precision=precision) as pc:
@@ -784,11 +802,8 @@ def realistic_leg(ctx, args, sample_clocks=True):
         e = error()
         out = {"value": job_rate(cmac_step, ctx.world, m * 1e-3), "unit": UNIT, "ms_per_step": m,
                "flush_ms": kf, "max_rel_err_I_vs_fp64": e}
-        if precision == "fp32":
-            out["roofline"] = ffma_roofline(cmac_step / max(kn, 1), kf, "flush_simt_kernel", kn,
-                                            (clocks or {}).get("sm_max_mhz"))
-        else:
-            out["roofline"] = tensor_roofline(cmac_step / max(kn, 1), kf, "flush_tc_drain2_kernel", kn, precision)
+        out["roofline"] = step_roofline(bytes_step, m, kf,
+                                        "flush_simt_kernel" if precision == "fp32" else "flush_tc_drain2_kernel", kn)
         return out
 
     fp16 = comparison("split_fp16", args.fp16_steps) if args.fp16_steps > 0 and args.precision == "split_bf16" else None
@@ -921,7 +936,8 @@ def batched_leg(ctx, args, sample_clocks=True):
             "max_rel_err_I_vs_fp64": worst, "error_sample": "2 (probe, pixel) series per partition, all energies",
             "eager_ms_per_step": eager_ms, "gpu_launches": launches, "contraction_launches_per_step": flushes,
             "clocks": clocks,
-            "roofline": tensor_roofline(cmac_step / max(k_n, 1), k_ms / max(k_n, 1), "flush_tc_drain2_kernel", k_n)}
+            "roofline": step_roofline(sum(s.P * s.Kx * s.Ky * (8.0 * s.T + 4.0 * s.Nw) for s in specs), ms,
+                                      k_ms / max(k_n, 1), "flush_tc_drain2_kernel", k_n)}
 
 
 # ----------------------------------------------------------------------------------------------
@@ -1011,7 +1027,7 @@ def diff_leg(ctx, args, sample_clocks=True):
     plan.close()
     del x, grad, I, S
     free_device()
-    fwd = ffma_roofline(cmac_fwd, fwd_ms, "flush_simt_kernel", k_n, (clocks or {}).get("sm_max_mhz"))
+    fwd = step_roofline(P * npix * (16.0 * T + 4.0 * Nw), ms, fwd_ms, "flush_simt_kernel", k_n)   # gradient written
     # the tensor-core adjoint call: its floor is the larger of the tensor time of its two
     # contractions and the HBM time of the bytes it must move (the gradient over the whole ROI of
     # every frame written once, the aperture rows' frames read once)
@@ -1115,16 +1131,15 @@ def thick_pipelined_leg(ctx, args, sample_clocks=True):
     plan.close()
     del ring, I, S
     free_device()
-    roof = tensor_roofline(cmac_step / max(k_per_step, 1), flush_ms, "flush_tc_drain2_kernel + conversion warps",
-                           k_per_step)
+    roof = step_roofline(spec.P * npix * (8.0 * T + 4.0 * Nw), ms, flush_ms, "flush_tc_drain2_kernel", k_per_step)
     return {"workload": name + "-pipelined-16", "value": job_rate(cmac_step, ctx.world, ms * 1e-3), "unit": UNIT,
             "ms_per_step": ms, "steps": args.steps, "warmup": args.warmup, "dtype": "bf16",
             "config": {"probes_per_step": spec.P, "segment_probes": H, "segments_per_step": n_seg,
                        "k_roi": f"{K}x{K} at ({rx}, {ry})", "T": T, "frames_per_push": Tc, "n_omega": Nw,
                        "plan_device_GB": round(info["device_bytes"] / 1e9, 1),
-                       "step": "per segment: reset + pushes (recorded) + finalize_async, which launches the "
-                               "previous segment's contraction with this segment's conversion in its extra "
-                               "warps; tacaw_drain after the last",
+                       "step": "per segment: reset + pushes (converted at once into the other staging area: "
+                               "band-limited blocks) + finalize_async, which launches the previous segment's "
+                               "contraction; tacaw_drain after the last",
                        "why_16": "two staging areas of 32 probes (2 x 137 GB) do not fit beside the input ring "
                                  "and I; two of 16 probes do"},
             "max_rel_err_I_vs_fp64": err, "error_sample": "16 (probe, pixel) series of the first and the last "
