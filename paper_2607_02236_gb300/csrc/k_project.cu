@@ -112,7 +112,8 @@ struct ProjSmem {
 // range's end) and undone in the contraction's epilogue.  A row that outgrows it has its staged
 // coefficients rescaled.
 // CHECK: frame components beyond 65504 / e.f16_scale set DEVERR_FP16_RANGE (split-FP16 plans).
-template <int B, int R, bool SPLIT, bool CHECK>
+// ONE: a launch of one entry, whose fields then are constants of the launch and not loads by index.
+template <int B, int R, bool SPLIT, bool CHECK, bool ONE>
 __global__ void __launch_bounds__(128, ProjSmem<B, R, SPLIT>::kCtas)
     project_group_kernel(const __grid_constant__ ProjGroup pg) {
     using SM = ProjSmem<B, R, SPLIT>;
@@ -133,7 +134,7 @@ __global__ void __launch_bounds__(128, ProjSmem<B, R, SPLIT>::kCtas)
     const int total = (int)pg.groups, step = (int)gridDim.x, first_group = (int)blockIdx.x;
     auto entry_of = [&](int rg) {
         int i = 0;
-        while (i + 1 < pg.n && rg >= pg.e[i + 1].group_begin) ++i;
+        while (!ONE && i + 1 < pg.n && rg >= pg.e[i + 1].group_begin) ++i;
         return i;
     };
     // The next stage to copy: block pk, stage pst of row group prg (entry pe); groups without a whole
@@ -146,10 +147,10 @@ __global__ void __launch_bounds__(128, ProjSmem<B, R, SPLIT>::kCtas)
     auto open_copy = [&]() {
         for (; prg < total; prg += step) {
             pe = entry_of(prg);
-            if (pg.e[pe].nblk > 0) break;
+            if (pg.e[ONE ? 0 : pe].nblk > 0) break;
         }
         if (prg < total) {
-            const ProjEntry &e = pg.e[pe];
+            const ProjEntry &e = pg.e[ONE ? 0 : pe];
             pm = (uint32_t)(prg - (int)e.group_begin) * 128u + threadIdx.x;
             const bool valid = (int64_t)pm < e.g.M;
             pbytes = valid ? 8 : 0;
@@ -162,7 +163,7 @@ __global__ void __launch_bounds__(128, ProjSmem<B, R, SPLIT>::kCtas)
     int put = 0;
     auto copy_stage = [&]() {
         if (prg < total) {
-            const ProjEntry &e = pg.e[pe];
+            const ProjEntry &e = pg.e[ONE ? 0 : pe];
             const int f0 = pk * B - e.c0;
             const int64_t pitch = e.g.pitch_frame;
             float2 *dst = ring + put * (2 * KP * 32);
@@ -207,7 +208,7 @@ __global__ void __launch_bounds__(128, ProjSmem<B, R, SPLIT>::kCtas)
     const float2 *mod_now = nullptr;
 #pragma unroll 1
     for (int rg = first_group; rg < total; rg += step) {
-        const ProjEntry &e = pg.e[entry_of(rg)];
+        const ProjEntry &e = pg.e[ONE ? 0 : entry_of(rg)];
         const uint32_t m = (uint32_t)(rg - (int)e.group_begin) * 128u + threadIdx.x;
         // (a block has more stages than the ring, so the copies are in this group: mu_next is its mean)
         const float2 mu = e.nblk > 0 ? mu_next : ((int64_t)m < e.g.M ? e.mu_hat[m] : make_float2(0.f, 0.f));
@@ -435,7 +436,7 @@ __global__ void __launch_bounds__(128) carry_group_kernel(const __grid_constant_
 template <int B, int R, bool SPLIT, bool CHECK>
 static cudaError_t launch_project_kernel(const ProjGroup &pg, cudaStream_t st) {
     using SM = ProjSmem<B, R, SPLIT>;
-    auto *kern = project_group_kernel<B, R, SPLIT, CHECK>;
+    auto *kern = pg.n == 1 ? project_group_kernel<B, R, SPLIT, CHECK, true> : project_group_kernel<B, R, SPLIT, CHECK, false>;
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

@@ -100,6 +100,35 @@ __global__ void __launch_bounds__(16 * TY) flush_simt_kernel(SimtArgs a, int n_j
         }
     }
     cp_async_wait<0>();
+    if (a.e.mode == FLUSH_FINAL && !a.e.has_prev && a.e.I_out && !a.e.Psi_out && !a.e.out_add) {
+        // intensities of a segment of one flush: tables read once a thread, pointers advanced by one pitch (the
+        // general epilogue below tests its mode and forms 64-bit addresses at each of the 8 Q elements)
+        float2 W[Q];
+        float B[Q];
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const int j = min(j0 + ty + TY * q, a.e.Nw - 1);
+            W[q] = __ldg(a.e.Wc + j);
+            B[q] = __ldg(a.e.bose + j);
+        }
+        const int64_t pitch = (int64_t)TY * a.e.npix;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const RowCtx row = make_row(a.e, m0 + tx + 16 * i);
+            if (!row.valid) continue;
+            float *out = a.e.I_out + row.out_base + (int64_t)(j0 + ty) * a.e.npix;
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                if (j0 + ty + TY * q < a.e.Nw) {
+                    const float pr = ar[i][q] - (row.dmu.x * W[q].x - row.dmu.y * W[q].y);
+                    const float pi = ai[i][q] - (row.dmu.x * W[q].y + row.dmu.y * W[q].x);
+                    *out = (pr * pr + pi * pi) * B[q] * a.e.out_scale;
+                }
+                out += pitch;
+            }
+        }
+        return;
+    }
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
         const int64_t m = m0 + tx + 16 * i;
