@@ -634,7 +634,7 @@ def thick_leg(ctx, args):
                        "window": spec.window, "detectors": D,
                        "precision": "split_bf16 plan: hi*hi + hi*lo + lo*hi, fp32 accumulate in tensor memory, hi*hi "
                                     "drained into fp32 registers (frames every "
-                                    f"{info['tc_drain_frames']}, block coefficients every 128 to 320 slots), fp64 "
+                                    f"{info['tc_drain_frames']}, block coefficients every 96 to 256 slots), fp64 "
                                     "phase; 64-frame blocks staged as fp16 hi + lo coefficients on the energies' band",
                        "value_counts": "rows x T x energies of the transform per step; band-limited staging and the "
                                        "two-level contraction reach the same result in fewer products",

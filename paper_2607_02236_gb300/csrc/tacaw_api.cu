@@ -245,9 +245,10 @@ TcPlanArgs tc_args(tacaw_plan_s *p, const Stream &s, const EpiArgs &e) {
     a.kbB0 = band ? s.stage_start / s.ring * (band->slots / p->bf) : s.stage_start / p->bf;
     a.bf = p->bf;
     a.stages = s.stages;
-    // coefficients sum more coherently than frames: chunks of at most 10 blocks keep the truncation of the
-    // tensor core's sums (the error grows with the chunk: 2.6e-6 at 16 blocks, 1.3e-6 at 8 on the scan)
-    a.drain_kb = band ? std::min(p->drain_kb, kBandDrainBlocks) : p->drain_kb;
+    // the truncation of the tensor core's sums grows with the products a chunk adds up coherently, so a chunk
+    // of coefficients stands for as many frames as one of frames (512 by default; on the scan of 2048 frames
+    // the error was 2.6e-6 at 16 blocks of coefficients, 1.3e-6 at the 8 that 512 frames fill)
+    a.drain_kb = band ? std::max(1, p->drain_kb * band->R / band->B) : p->drain_kb;
     a.A_hi = s.A_hi;
     a.A_lo = s.A_lo;
     a.B_hi = band ? band->B_hi : s.B_hi;
@@ -268,7 +269,7 @@ TcPlanArgs tc_args(tacaw_plan_s *p, const Stream &s, const EpiArgs &e) {
         a.A_lo = s.A_lo + 2 * (size_t)band->z_begin() * (size_t)s.M_pad;
         a.a_group = 4 * (int64_t)band->z_slots * s.M_pad;
         a.row_unit *= (float)(1 << band->z_shift());
-        a.drain_kb = std::min(a.drain_kb, 4);   // (the first level's sums are truncated too)
+        a.drain_kb = std::min(p->drain_kb, kBandDrainBlocks);
     }
     a.err = p->d_err;
     a.trace = nullptr;
@@ -297,7 +298,7 @@ tacaw_status launch_first_level(tacaw_plan_s *p, const Stream *const *streams, i
         a.n_sb = (a.total_kb + a.n_kb - 1) / a.n_kb;
         a.bf = p->bf;
         a.stages = s.stages;
-        a.drain_kb = kBandDrainBlocks;
+        a.drain_kb = std::max(1, p->drain_kb * b.R / b.B);
         a.A_hi = s.A_hi;
         a.A_lo = s.A_lo;
         a.B_hi = b.T_hi;
@@ -841,7 +842,8 @@ tacaw_status launch_pending(tacaw_plan_s *p, const Stream *conv, cudaStream_t st
     TraceRange trace_range(conv ? "contraction (tensor cores) with the next conversion" : "contraction (tensor cores)");
     tacaw_plan_s::Pending &q = p->pend;
     Stream &ps = q.snap;
-    CU_CHECK(p, launch_mean_residual(ps.M, ps.T, ps.d.subtract_mean, ps.sum_res, ps.dmu, p->f16_scale, st),
+    CU_CHECK(p, launch_mean_residual(ps.M, ps.T, ps.d.subtract_mean, ps.sum_res, ps.shift_mean ? ps.mu_hat : nullptr, ps.dmu,
+                                     p->f16_scale, st),
              "mean residual");
     p->launches++;
     TcPlanArgs a = tc_args(p, ps, epi_args(p, ps, FLUSH_FINAL, q.I, q.Psi));
@@ -935,7 +937,8 @@ tacaw_status finalize_impl(tacaw_plan_t p, float *d_I, float *d_S, void *d_Psi, 
     if (!p->in_place)
         for (auto &s : p->s) {
             if (p->us[s.user].N > 1) continue;
-            CU_CHECK(p, launch_mean_residual(s.M, s.T, s.d.subtract_mean, s.sum_res, s.dmu, p->f16_scale, st),
+            CU_CHECK(p, launch_mean_residual(s.M, s.T, s.d.subtract_mean, s.sum_res, s.shift_mean ? s.mu_hat : nullptr, s.dmu,
+                                          p->f16_scale, st),
                      "mean residual");
             p->launches++;
         }
@@ -1060,7 +1063,7 @@ tacaw_status push_internal(tacaw_plan_s *p, Stream &s, const float2 *frames, int
         tacaw_status r = flush_due(p, st);
         if (r != TACAW_OK) return r;
     }
-    if (s.pushed == 0 && s.d.subtract_mean) {
+    if (s.pushed == 0 && s.removes_mean()) {
         CU_CHECK(p, launch_mean(g, n_frames, s.mu_hat, st), "provisional mean");
         p->launches++;
     }
@@ -1132,7 +1135,8 @@ tacaw_status push_internal(tacaw_plan_s *p, Stream &s, const float2 *frames, int
 // and make the lane ready for its next segment.
 tacaw_status finish_segment(tacaw_plan_s *p, UserStream &u, Stream &s, cudaStream_t st) {
     if (!p->in_place) {
-        CU_CHECK(p, launch_mean_residual(s.M, s.T, s.d.subtract_mean, s.sum_res, s.dmu, p->f16_scale, st),
+        CU_CHECK(p, launch_mean_residual(s.M, s.T, s.d.subtract_mean, s.sum_res, s.shift_mean ? s.mu_hat : nullptr, s.dmu,
+                                          p->f16_scale, st),
                  "mean residual");
         p->launches++;
     }
@@ -1641,7 +1645,7 @@ tacaw_status tacaw_push_frames_group(tacaw_plan_t p, int n, const int *stream_id
             banded[k] = 0;
             ids.push_back(k);
             const FrameGeom g = push_geom(s, static_cast<const float2 *>(d_frames[k]));
-            if (s.pushed == 0 && s.d.subtract_mean) {
+            if (s.pushed == 0 && s.removes_mean()) {
                 CU_CHECK(p, launch_mean(g, n_frames[k], s.mu_hat, st), "provisional mean");
                 p->launches++;
             }
@@ -1669,7 +1673,7 @@ tacaw_status tacaw_push_frames_group(tacaw_plan_t p, int n, const int *stream_id
             e.sum_res = s.sum_res;
             e.A_hi = s.A_hi;
             e.A_lo = s.A_lo;
-            if (s.pushed == 0 && s.d.subtract_mean) {
+            if (s.pushed == 0 && s.removes_mean()) {
                 CU_CHECK(p, launch_mean(e.g, e.n, s.mu_hat, st), "provisional mean");
                 p->launches++;
             }

@@ -353,6 +353,7 @@ tacaw_status build_band_forms(tacaw_plan_s *p, Stream &s, int64_t room_bytes, Ba
         CU_CHECK(p, launch_band_response(ta, ba, d_resp, st), "band response");
         CU_CHECK(p, launch_band_twiddles(ta, ba, d_resp, b.B_hi, b.B_lo, b.B32, st), "band twiddles");
         s.band[s.n_band++] = b;
+        s.shift_mean = !s.d.subtract_mean && !p->f16;   // (split FP16 checks the range of the frames as they are)
     }
     return TACAW_OK;
 }

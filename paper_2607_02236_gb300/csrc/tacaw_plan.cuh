@@ -41,7 +41,7 @@ struct BandForm {
     }
 };
 constexpr int kBandForms = 2;
-constexpr int kBandDrainBlocks = 10;   // staging blocks per drained H chunk on band-limited forms
+constexpr int kBandDrainBlocks = 3;   // staging blocks per drained H chunk of a second level (tacaw_api.cu)
 
 struct Stream {
     tacaw_stream_desc d{};
@@ -104,6 +104,11 @@ struct Stream {
     BandForm band[kBandForms];
     int n_band = 0;
     int form = -1;
+    // the provisional mean leaves the frames although the stream keeps its mean; the last flush adds
+    // mu_hat W(E) back.  Streams with band-limited forms: their coefficients' sums of an elastic line a
+    // hundred times the signal were 2.0e-6 of the intensities off, the frames' 1.1e-6.
+    bool shift_mean = false;
+    bool removes_mean() const { return d.subtract_mean || shift_mean; }
     // staged slots of the ring: frames, or the coefficients of its blocks (whole ones, and at the
     // segment's end a short one)
     int ring_slots() const {
