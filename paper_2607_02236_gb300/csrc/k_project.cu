@@ -10,8 +10,8 @@
 //
 // with the window and the shift to the band's centre f_c in m.  The contraction then runs over
 // coefficients as it runs over frames (32 staged slots to a block of its rows, its own twiddle table),
-// with R / B of the work, and the staged rows are R / B as long.  DESIGN notes beside the tables
-// (k_tables.cu) give the reconstruction error; R is chosen for it at plan creation.
+// with R / B of the work, and the staged rows are R / B as long.  k_tables.cu holds the expansion, and
+// tacaw_band.cu chooses R at plan creation for a reconstruction error of 1e-7 (kBandTol).
 //
 // One thread per row (probe, ROI pixel); a CTA takes groups of 128 rows of the push, all blocks of a group
 // one after another, with the frames of the next stages (4 or 8 frames each) in flight into each warp's ring
