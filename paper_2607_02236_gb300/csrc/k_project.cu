@@ -176,13 +176,13 @@ __global__ void __launch_bounds__(128, ProjSmem<B, R, SPLIT>::kCtas)
                     pb -= pitch;
                 }
             } else {
-                // frames before the push are in the carry; frames past the segment's end are zero
+                // frames before the push are in the carry; frames past the segment's end are zero, as padding
+                // rows are, whose carry nobody writes
 #pragma unroll
                 for (int i = 0; i < KP; ++i) {
                     const int u = KP * pst + i, v = B - 1 - u, f = f0 + u, g = f0 + v;
-                    proj_copy(dst + i * 32, f < 0 ? e.carry + (int64_t)u * e.M_pad + pm : pa, f < 0 ? 8 : (f < e.n ? pbytes : 0));
-                    proj_copy(dst + (KP + i) * 32, g < 0 ? e.carry + (int64_t)v * e.M_pad + pm : pb,
-                              g < 0 ? 8 : (g < e.n ? pbytes : 0));
+                    proj_copy(dst + i * 32, f < 0 ? e.carry + (int64_t)u * e.M_pad + pm : pa, f < e.n ? pbytes : 0);
+                    proj_copy(dst + (KP + i) * 32, g < 0 ? e.carry + (int64_t)v * e.M_pad + pm : pb, g < e.n ? pbytes : 0);
                     pa += pitch;
                     pb -= pitch;
                 }

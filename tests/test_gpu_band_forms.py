@@ -1,0 +1,111 @@
+"""Band-limited staging where its forms are picked: rows enough for the rule to choose blocks of a known
+length (read back from the plan's checkpoint, which records the form of each ring), pushes that leave
+blocks unfinished, and plans whose segments change form.  Sampled pixels are held against the FP64
+oracle at the suite's 1e-5 of the peak."""
+import numpy as np
+import pytest
+
+import oracle
+from tests.helpers import rel_err_peak
+
+pytestmark = pytest.mark.gpu
+
+TOL = 1e-5
+KX, KY = 131, 127          # 16 637 rows: 3 of the last row tile's 128 are padding
+ROWS = KX * KY
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    from paper_2607_02236_gb300 import build
+    build.build_all()
+
+
+def config(T, nw, E_max, **kw):
+    from paper_2607_02236_gb300 import DetectorConfig, StreamConfig
+    base = dict(n_probes=1, kx=KX, ky=KY, T=T, dt_fs=5.0, pitch_row=KX, pitch_frame=ROWS, pitch_probe=ROWS,
+                E_meV=list(np.arange(nw) * (E_max / nw)), detectors=[DetectorConfig(r_out=5.0)])
+    base.update(kw)
+    return StreamConfig(**base)
+
+
+def waves(T, seed, E_max=120.0, elastic=1.0, rows=ROWS):
+    """[T, rows] complex64 on the GPU: an elastic part, five lines inside the energies, noise."""
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    t = torch.arange(T, device="cuda", dtype=torch.float64)
+    E = E_max * (0.1 + 0.8 * torch.rand(5, device="cuda", dtype=torch.float64, generator=g))
+    line = torch.exp(2j * np.pi * torch.frac(t[:, None] * (E * (5e-3 / 4.135667696)))).to(torch.complex64)
+    amp = torch.polar(0.05 + 0.05 * torch.rand(5, rows, device="cuda", generator=g),
+                      2 * np.pi * torch.rand(5, rows, device="cuda", generator=g))
+    fr = line @ amp
+    fr += elastic * torch.polar(torch.ones(rows, device="cuda"), 2 * np.pi * torch.rand(rows, device="cuda", generator=g))
+    torch.view_as_real(fr).add_(torch.randn(T, rows, 2, device="cuda", generator=g), alpha=1e-4)
+    return fr
+
+
+def at(fr, t):
+    return fr.data_ptr() + t * fr.stride(0) * 8
+
+
+def push_all(plan, fr, sizes, a=0, b=None, push=None):
+    """Frames [a, b) in pushes of the sizes in turn."""
+    b = fr.shape[0] if b is None else b
+    i = 0
+    while a < b:
+        n = min(sizes[i % len(sizes)], b - a)
+        (push or plan.push)(0, at(fr, a), n)
+        a += n
+        i += 1
+
+
+def ring_form(plan, stream=0):
+    """Block length of the form the stream's ring holds (0: frames), from its checkpoint."""
+    rec = plan.save_state()[48 + 48 * stream:48 + 48 * (stream + 1)]
+    return int(rec[44:48].view(np.int32)[0])
+
+
+def finish(plan, psi=False):
+    """(I, Psi) [nw, rows] of the finished segment."""
+    import torch
+    n = plan.info()["I_elems"]
+    I = torch.full((n,), -1.0, device="cuda")
+    S = torch.empty(max(1, plan.info()["S_elems"]), device="cuda")
+    P = torch.zeros(n, dtype=torch.complex64, device="cuda") if psi else None
+    plan.finalize(I, S, P)
+    return I.cpu().numpy().reshape(-1, ROWS), P.cpu().numpy().reshape(-1, ROWS) if psi else None
+
+
+PIX = np.r_[0:16, 1000:16000:997, ROWS - 16:ROWS]
+
+
+def assert_exact(I, fr, cfg, Psi=None):
+    kw = dict(window_kind=cfg.window, window_param=cfg.window_param, E_meV=cfg.E_meV, subtract_mean=cfg.subtract_mean)
+    psi, want = oracle.forward_pixels(fr[:, PIX].cpu().numpy(), **kw)
+    e = rel_err_peak(I[:, PIX], want)
+    assert e <= TOL, e
+    if Psi is not None:
+        e = rel_err_peak(Psi[:, PIX], psi)
+        assert e <= TOL, e
+
+
+@pytest.mark.parametrize("precision", ["split_fp16", "split_bf16"])
+def test_unfinished_blocks_after_another_form(precision):
+    """A segment of plain frames, then one of 16-frame pushes into blocks of 64: three of four pushes only
+    carry, and the place of the carry holds the first segment's staged frames.  Rows past the last one take
+    no part: no range error, and the results of a plan's first segment."""
+    from paper_2607_02236_gb300 import TacawPlan
+    cfg = config(1024, 1000, 150.0)
+    fr = waves(1024, 3)
+    with TacawPlan([cfg], precision=precision) as plan:
+        push_all(plan, fr, [8])
+        finish(plan)
+        plan.reset()
+        push_all(plan, fr, [16], 0, 48)
+        assert ring_form(plan) == 64
+        push_all(plan, fr, [16], 48)
+        I, _ = finish(plan)
+    assert_exact(I, fr, cfg)
+    with TacawPlan([cfg], precision=precision) as plan:
+        push_all(plan, fr, [16])
+        assert np.array_equal(finish(plan)[0], I)
