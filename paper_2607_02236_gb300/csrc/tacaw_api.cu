@@ -1615,15 +1615,15 @@ tacaw_status tacaw_push_frames_group(tacaw_plan_t p, int n, const int *stream_id
     for (int i = 0; i < n; ++i) {
         const UserStream &u = p->us[stream_ids[i]];
         Stream &s = p->s[u.first];
-        // pushes that lie in the ring and take one of its band-limited forms
-        if (u.N <= 1 && !p->in_place && !p->pipe && u.pushed >= u.skip && !s.due && s.staged + n_frames[i] <= s.ring) {
-            if (s.staged == 0) s.form = choose_form(p, s, n_frames[i]);
-            banded[i] = s.form >= 0;
-            if (banded[i]) continue;
-        }
-        const bool ok = split && u.N <= 1 && u.pushed >= u.skip && !s.due && s.staged + n_frames[i] <= s.ring &&
-                        convert_split_groupable(p->bf, s.staged, n_frames[i]);
-        if (ok) {
+        // whole-stream pushes that lie in the ring; a pipelined plan (of one stream) goes by the single push,
+        // which knows whether its segment's frames are recorded or converted
+        const bool in_ring = u.N <= 1 && !p->in_place && !p->pipe && u.pushed >= u.skip && !s.due &&
+                             s.staged + n_frames[i] <= s.ring;
+        // the form is the ring's: its first push picks it, later ones continue it
+        if (in_ring && s.staged == 0) s.form = choose_form(p, s, n_frames[i]);
+        banded[i] = in_ring && s.form >= 0;
+        if (banded[i]) continue;
+        if (in_ring && split && convert_split_groupable(p->bf, s.staged, n_frames[i])) {
             grouped.push_back(i);
         } else {
             c = push_user(p, stream_ids[i], static_cast<const float2 *>(d_frames[i]), n_frames[i], st);

@@ -109,3 +109,37 @@ def test_unfinished_blocks_after_another_form(precision):
     with TacawPlan([cfg], precision=precision) as plan:
         push_all(plan, fr, [16])
         assert np.array_equal(finish(plan)[0], I)
+
+
+@pytest.mark.parametrize("nw,ring", [(1000, 64), (100, 0)])
+def test_pipelined_plan_single_and_group_pushes(nw, ring):
+    """A pipelined plan takes single and group pushes of one segment: the first segment's converted at push
+    time (into blocks of 64 frames at 1000 energies, as plain frames at 100), the second's while the first's
+    contraction is pending.  The bits are those of an unpipelined plan's single pushes."""
+    import torch
+    from paper_2607_02236_gb300 import TacawPlan
+    cfg = config(1024, nw, 150.0)
+    frs = [waves(1024, 5), waves(1024, 6)]
+    st = torch.cuda.current_stream()
+    outs = []
+    for pipe in (False, True):
+        with TacawPlan([cfg], precision="split_bf16") as plan:
+            plan.set_pipelined_segments(pipe)
+            Is = [torch.full((plan.info()["I_elems"],), -1.0, device="cuda") for _ in frs]
+            for k, fr in enumerate(frs):
+                plan.reset(st)
+                for i, t in enumerate(range(0, 1024, 32)):
+                    if pipe and i % 3:
+                        plan.push_group([0], [at(fr, t)], [32], st)
+                    else:
+                        plan.push(0, at(fr, t), 32, st)
+                    if k == 0 and i == 1:
+                        assert ring_form(plan) == ring
+                plan.finalize_async(Is[k], None, None, st)
+            if pipe:
+                plan.drain(st)
+            plan.check_errors(st)
+            outs.append([I.cpu().numpy().reshape(-1, ROWS) for I in Is])
+    for k, fr in enumerate(frs):
+        assert np.array_equal(outs[0][k], outs[1][k])
+        assert_exact(outs[0][k], fr, cfg)
