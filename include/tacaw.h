@@ -365,7 +365,8 @@ tacaw_status tacaw_reset(tacaw_plan_t plan, void *stream);
  * resume by recomputing every batch not marked finished: Sec. II.B, batch dispatching).  The
  * accumulation is a sum over the pushed frames, so between two pushes a plan's progress is a
  * few buffers, and a plan created from the same descriptor that loads them continues where the
- * saving plan stopped: the same later pushes give bit-identical results.
+ * saving plan stopped: the same later pushes give bit-identical results (to rounding where the two
+ * plans' memory at creation left room for different band-limited forms).
  * tacaw_state_size: bytes of a checkpoint of the plan as it is now (after the pushes enqueued
  *   so far): a 48-byte header, 48 bytes per internal stream (Welch lanes count one each) and 8
  *   per stream, then the device sections.  Per internal stream: the provisional mean (8 bytes a
@@ -383,9 +384,10 @@ tacaw_status tacaw_reset(tacaw_plan_t plan, void *stream);
  *   (precision, accumulators, K_stage, block frames, ROI, energies, window, time step, mean
  *   subtraction and Welch segmentation must give the same layout; energy tiles and other
  *   tuning may differ).  It replaces the plan's segment in progress, finalized or not; the
- *   copies run on `stream` and the call returns when they are done.  INVALID_ARG, with the plan
- *   unchanged, for bytes that are not a checkpoint, are truncated or corrupted, or were saved
- *   by another configuration.
+ *   copies run on `stream` and the call returns when they are done.  A ring saved in a band-limited
+ *   form that the plan had no room for has that form's tables built (OOM if they do not fit).
+ *   INVALID_ARG, with the plan unchanged, for bytes that are not a checkpoint, are truncated or
+ *   corrupted, or were saved by another configuration.
  * STATE for tacaw_state_size and tacaw_save_state: a finalized segment (nothing to resume), a
  *   deferred contraction (pipelined segments: tacaw_drain first, also before a restore), or,
  *   with frames_in_place, pushed frames not yet contracted (the plan holds only their

@@ -375,7 +375,7 @@ __global__ void zero_tail_split_kernel(int64_t M_pad, int staged, int bf, uint32
     }
 }
 
-__global__ void mean_residual_kernel(int64_t M, int T, int sub, const double2 *sum_res, const float2 *added_back,
+__global__ void mean_residual_kernel(int64_t M, int T, int sub, const double2 *sum_res, const float2 *mu_hat,
                                      float2 *dmu, double sc) {
     int64_t m = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (m >= M) return;
@@ -383,7 +383,7 @@ __global__ void mean_residual_kernel(int64_t M, int T, int sub, const double2 *s
         const double2 s = sum_res[m];
         dmu[m] = make_float2((float)(sc * s.x / T), (float)(sc * s.y / T));
     } else {
-        const float2 mu = added_back ? added_back[m] : make_float2(0.f, 0.f);
+        const float2 mu = mu_hat[m];
         dmu[m] = make_float2((float)(-sc * mu.x), (float)(-sc * mu.y));
     }
 }
@@ -489,9 +489,9 @@ cudaError_t launch_zero_tail_split(int64_t M_pad, int staged, int bf, __nv_bfloa
     return cudaGetLastError();
 }
 
-cudaError_t launch_mean_residual(int64_t M, int T, int subtract_mean, const double2 *sum_res, const float2 *added_back,
+cudaError_t launch_mean_residual(int64_t M, int T, int subtract_mean, const double2 *sum_res, const float2 *mu_hat,
                                  float2 *dmu, float scale, cudaStream_t st) {
-    mean_residual_kernel<<<blocks_for(M, 256), 256, 0, st>>>(M, T, subtract_mean, sum_res, added_back, dmu, (double)scale);
+    mean_residual_kernel<<<blocks_for(M, 256), 256, 0, st>>>(M, T, subtract_mean, sum_res, mu_hat, dmu, (double)scale);
     return cudaGetLastError();
 }
 

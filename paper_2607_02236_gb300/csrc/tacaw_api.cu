@@ -842,8 +842,7 @@ tacaw_status launch_pending(tacaw_plan_s *p, const Stream *conv, cudaStream_t st
     TraceRange trace_range(conv ? "contraction (tensor cores) with the next conversion" : "contraction (tensor cores)");
     tacaw_plan_s::Pending &q = p->pend;
     Stream &ps = q.snap;
-    CU_CHECK(p, launch_mean_residual(ps.M, ps.T, ps.d.subtract_mean, ps.sum_res, ps.shift_mean ? ps.mu_hat : nullptr, ps.dmu,
-                                     p->f16_scale, st),
+    CU_CHECK(p, launch_mean_residual(ps.M, ps.T, ps.d.subtract_mean, ps.sum_res, ps.mu_hat, ps.dmu, p->f16_scale, st),
              "mean residual");
     p->launches++;
     TcPlanArgs a = tc_args(p, ps, epi_args(p, ps, FLUSH_FINAL, q.I, q.Psi));
@@ -937,8 +936,7 @@ tacaw_status finalize_impl(tacaw_plan_t p, float *d_I, float *d_S, void *d_Psi, 
     if (!p->in_place)
         for (auto &s : p->s) {
             if (p->us[s.user].N > 1) continue;
-            CU_CHECK(p, launch_mean_residual(s.M, s.T, s.d.subtract_mean, s.sum_res, s.shift_mean ? s.mu_hat : nullptr, s.dmu,
-                                          p->f16_scale, st),
+            CU_CHECK(p, launch_mean_residual(s.M, s.T, s.d.subtract_mean, s.sum_res, s.mu_hat, s.dmu, p->f16_scale, st),
                      "mean residual");
             p->launches++;
         }
@@ -1135,8 +1133,7 @@ tacaw_status push_internal(tacaw_plan_s *p, Stream &s, const float2 *frames, int
 // and make the lane ready for its next segment.
 tacaw_status finish_segment(tacaw_plan_s *p, UserStream &u, Stream &s, cudaStream_t st) {
     if (!p->in_place) {
-        CU_CHECK(p, launch_mean_residual(s.M, s.T, s.d.subtract_mean, s.sum_res, s.shift_mean ? s.mu_hat : nullptr, s.dmu,
-                                          p->f16_scale, st),
+        CU_CHECK(p, launch_mean_residual(s.M, s.T, s.d.subtract_mean, s.sum_res, s.mu_hat, s.dmu, p->f16_scale, st),
                  "mean residual");
         p->launches++;
     }

@@ -258,7 +258,8 @@ std::vector<double> choose_levels(const Stream &s, BandForm &b, std::vector<doub
 
 namespace tacaw {
 
-tacaw_status build_band_forms(tacaw_plan_s *p, Stream &s, int64_t room_bytes, BandCache &cache, cudaStream_t st) {
+tacaw_status build_band_forms(tacaw_plan_s *p, Stream &s, int64_t room_bytes, BandCache &cache, cudaStream_t st,
+                              int only) {
     const bool split = p->prec == TACAW_PREC_SPLIT_BF16;
     if (p->in_place || (split && p->bf != 32) || s.T < kBandMinT) return TACAW_OK;
     const double dt_ps = s.d.dt_fs * 1e-3;
@@ -272,6 +273,7 @@ tacaw_status build_band_forms(tacaw_plan_s *p, Stream &s, int64_t room_bytes, Ba
     if (!(beta < 0.5)) return TACAW_OK;   // no form pays (R / B near 1)
     const double fc = 0.5 * (lo + hi) * dt_ps / kPlanck_meV_ps;
     for (int B : {32, 64, 128}) {
+        if (only && B != only) continue;
         if (!project_shape_ok(B, 8, split) || (s.needs_acc && s.ring % B)) continue;   // flushes end between blocks
         int R = 0;
         const std::vector<double> &basis = cache.basis(B, std::max(beta, 1e-6), 8, 48, &R);

@@ -323,9 +323,9 @@ cudaError_t launch_convert_fp32(const FrameGeom &g, int n, int s0, int64_t M_pad
 cudaError_t launch_frame_table(const float2 **table, const float2 *base, int64_t pitch_frame, int n, cudaStream_t st);
 cudaError_t launch_zero_tail_split(int64_t M_pad, int staged, int bf, __nv_bfloat16 *A_hi, __nv_bfloat16 *A_lo,
                                    int swz, cudaStream_t st);
-// dmu = scale * (mu - mu_hat) (scale: the split-FP16 operand scale, else 1); with the mean kept
-// -scale * mu_hat (added_back: the provisional mean that left the frames), or 0 (null)
-cudaError_t launch_mean_residual(int64_t M, int T, int subtract_mean, const double2 *sum_res, const float2 *added_back,
+// dmu = scale * (mu - mu_hat) (scale: the split-FP16 operand scale, else 1); with the mean kept -scale * mu_hat:
+// every conversion takes mu_hat out of the frames, so what it holds is added back, zeros where no mean was taken
+cudaError_t launch_mean_residual(int64_t M, int T, int subtract_mean, const double2 *sum_res, const float2 *mu_hat,
                                  float2 *dmu, float scale, cudaStream_t st);
 
 // Push conversion into band-limited block coefficients (k_project.cu).  One push of one stream:

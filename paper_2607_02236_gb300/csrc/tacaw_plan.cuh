@@ -105,7 +105,8 @@ struct Stream {
     int n_band = 0;
     int form = -1;
     // the provisional mean leaves the frames although the stream keeps its mean; the last flush adds
-    // mu_hat W(E) back.  Streams with band-limited forms: their coefficients' sums of an elastic line a
+    // mu_hat W(E) back, which it does for whatever mu_hat holds (a restored segment's may come from a plan
+    // with other forms).  Streams with band-limited forms: their coefficients' sums of an elastic line a
     // hundred times the signal were 2.0e-6 of the intensities off, the frames' 1.1e-6.
     bool shift_mean = false;
     bool removes_mean() const { return d.subtract_mean || shift_mean; }
@@ -236,8 +237,9 @@ struct BandCache {
     const std::vector<double> &basis(int B, double beta, int min_rank, int max_rank, int *rank);
 };
 // Builds the band-limited staging forms that pay for stream s (tacaw_band.cu), within room_bytes of
-// device memory; a stream without any keeps staging frames.
-tacaw_status build_band_forms(tacaw_plan_s *p, Stream &s, int64_t room_bytes, BandCache &cache, cudaStream_t st);
+// device memory; a stream without any keeps staging frames.  only: just the form with blocks of that many frames.
+tacaw_status build_band_forms(tacaw_plan_s *p, Stream &s, int64_t room_bytes, BandCache &cache, cudaStream_t st,
+                              int only = 0);
 // The staging form a ring takes whose first push has n frames (-1: frames).
 int choose_form(const tacaw_plan_s *p, const Stream &s, int n);
 // Table arguments of stream s after its tables were built.

@@ -22,7 +22,8 @@ namespace {
 // everything else a plan holds (tables, detector lists) follows from its descriptor, which the
 // fingerprint ties to the checkpoint.
 constexpr uint64_t kStateMagic = 0x314B435741434154ULL;   // the bytes "TACAWCK1"
-constexpr uint32_t kStateVersion = 1;
+// Version 1: before StreamCounters::form (zero there), when a kept mean stayed in the frames (mu_hat zero); read as well.
+constexpr uint32_t kStateVersion = 2;
 
 struct StateHeader {
     uint64_t magic;
@@ -62,7 +63,8 @@ struct Fnv {
 // What the saved buffers' contents and layout depend on: precision, accumulators, staging
 // geometry, the frames' ROI and the arithmetic of the tables (energies, window, time step,
 // mean subtraction), and the Welch segmentation.  Tuning that does not change a saved layout
-// (energy tiles, pipeline depth, CTA caps) is left out.
+// (energy tiles, pipeline depth, CTA caps) is left out, and so are the band-limited forms a plan
+// has (they depend on the memory left at its creation): each ring's own form is in its counters.
 uint64_t plan_fingerprint(const tacaw_plan_s *p) {
     Fnv f;
     f.val(p->prec);
@@ -222,7 +224,7 @@ tacaw_status check_counters(const tacaw_plan_s *p, const std::vector<StreamCount
                         k.stage_start >= 0 && k.stage_start + k.staged == k.pushed && k.flushes >= 0 &&
                         k.flushes <= k.stage_start && (s.needs_acc || k.flushes == 0) &&
                         (!p->in_place || k.staged == 0) && (k.due == 0 || (k.due == 1 && k.staged == s.ring)) &&
-                        (k.form == 0 || (k.staged > 0 && band_of(s, k.form) >= 0)) &&
+                        (k.form == 0 || (k.staged > 0 && (k.form == 32 || k.form == 64 || k.form == 128))) &&
                         k.seg >= s.lane && (k.seg - s.lane) % u.lanes == 0 &&
                         k.seg < s.lane + (int64_t)u.lanes * (u.N + 1);
         if (!ok) return fail(TACAW_ERR_INVALID_ARG, "checkpoint: counters of stream %zu are inconsistent", i);
@@ -304,8 +306,8 @@ tacaw_status tacaw_restore_state(tacaw_plan_t p, const void *h_state, int64_t by
         return fail(TACAW_ERR_INVALID_ARG, "checkpoint: %lld bytes is too short", (long long)bytes);
     std::memcpy(&h, in, sizeof h);
     if (h.magic != kStateMagic) return fail(TACAW_ERR_INVALID_ARG, "checkpoint: not a plan checkpoint");
-    if (h.version != kStateVersion)
-        return fail(TACAW_ERR_INVALID_ARG, "checkpoint: version %u, this library reads %u", h.version, kStateVersion);
+    if (h.version < 1 || h.version > kStateVersion)
+        return fail(TACAW_ERR_INVALID_ARG, "checkpoint: version %u, this library reads 1 to %u", h.version, kStateVersion);
     if (h.n_streams != p->s.size() || h.n_user != p->us.size() || h.fingerprint != plan_fingerprint(p))
         return fail(TACAW_ERR_INVALID_ARG, "checkpoint: saved by a plan of another configuration");
     if (h.total_bytes > bytes)
@@ -326,10 +328,20 @@ tacaw_status tacaw_restore_state(tacaw_plan_t p, const void *h_state, int64_t by
     if (f.h != h.counters_hash) return fail(TACAW_ERR_INVALID_ARG, "checkpoint: counter records corrupted");
     c = check_counters(p, cnt, uc);
     if (c != TACAW_OK) return c;
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    // a ring in a form whose tables this plan had no room for at its creation: they are built now
+    BandCache bases;
+    for (size_t i = 0; i < p->s.size(); ++i) {
+        if (cnt[i].form == 0 || band_of(p->s[i], cnt[i].form) >= 0) continue;
+        c = build_band_forms(p, p->s[i], INT64_MAX, bases, st, cnt[i].form);
+        if (c != TACAW_OK) return c;
+        if (band_of(p->s[i], cnt[i].form) < 0)
+            return fail(TACAW_ERR_OOM, "checkpoint: no memory for the tables of stream %zu's blocks of %d frames", i,
+                        cnt[i].form);
+    }
     if (state_total(p, cnt) != h.total_bytes)
         return fail(TACAW_ERR_INVALID_ARG, "checkpoint: section sizes do not match its counters");
     // the checkpoint is this plan's: load the device sections, then the counters
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
     for (const StateSection &x : state_sections(p, cnt)) {
         CU_CHECK(p, cudaMemcpyAsync(x.dev, in + off, x.bytes, cudaMemcpyHostToDevice, st), "checkpoint copy");
         off += x.bytes;

@@ -143,3 +143,61 @@ def test_pipelined_plan_single_and_group_pushes(nw, ring):
     for k, fr in enumerate(frs):
         assert np.array_equal(outs[0][k], outs[1][k])
         assert_exact(outs[0][k], fr, cfg)
+
+
+def no_room(cfg, k_stage, **kw):
+    """Plan arguments whose budget is what the plan needs without any form's tables."""
+    import re
+    from paper_2607_02236_gb300 import TacawError, TacawPlan
+    with pytest.raises(TacawError) as e:
+        TacawPlan([cfg], k_stage=k_stage, hbm_budget_bytes=1, **kw)
+    return dict(kw, k_stage=k_stage, hbm_budget_bytes=int(re.search(r"needs (\d+) bytes", str(e.value)).group(1)))
+
+
+@pytest.mark.parametrize("mean", [False, True])
+@pytest.mark.parametrize("ring,sizes", [(0, [8]), (64, [64, 16])])
+@pytest.mark.parametrize("saver", ["with forms", "without"])
+def test_checkpoint_between_plans_with_and_without_forms(saver, ring, sizes, mean):
+    """A plan with memory for band-limited forms and one without take each other's checkpoints, also where the
+    stream keeps its mean (which a plan with forms takes out of the frames and adds back) and where the ring
+    holds coefficients (the loader then builds that form's tables)."""
+    from paper_2607_02236_gb300 import TacawPlan
+    cfg = config(1024, 1000, 150.0, subtract_mean=mean)
+    fr = waves(1024, 8)
+    plans = [dict(precision="split_bf16", k_stage=1024), no_room(cfg, 1024, precision="split_bf16")]
+    if saver == "without":
+        plans.reverse()
+    with TacawPlan([cfg], **plans[0]) as A:
+        push_all(A, fr, sizes, 0, 144)
+        assert ring_form(A) == (ring if saver == "with forms" else 0)
+        state = A.save_state()
+    with TacawPlan([cfg], **plans[1]) as B:
+        push_all(B, fr, [64], 0, 64)          # a segment in progress that the checkpoint replaces
+        assert ring_form(B) == (0 if saver == "with forms" else 64)
+        B.restore_state(state)
+        push_all(B, fr, [64], 144)
+        I, _ = finish(B)
+    assert_exact(I, fr, cfg)
+
+
+def test_checkpoint_versions():
+    """Checkpoints of the version before forms (plain frames, kept mean left in them) are read; later ones not."""
+    from paper_2607_02236_gb300 import TacawError, TacawPlan
+    cfg = config(256, 64, 120.0)
+    fr = waves(256, 9)
+    with TacawPlan([cfg], precision="split_bf16") as plan:
+        push_all(plan, fr, [32], 0, 96)
+        state = plan.save_state()
+        push_all(plan, fr, [32], 96)
+        want, _ = finish(plan)
+        version = int(state[8:12].view(np.uint32)[0])
+        assert version == 2
+        for v, ok in ((1, True), (2, True), (3, False), (0, False)):
+            state[8:12] = np.frombuffer(np.uint32(v).tobytes(), np.uint8)
+            if not ok:
+                with pytest.raises(TacawError, match="version"):
+                    plan.restore_state(state)
+                continue
+            plan.restore_state(state)
+            push_all(plan, fr, [32], 96)
+            assert np.array_equal(finish(plan)[0], want)
