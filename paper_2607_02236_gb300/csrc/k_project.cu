@@ -69,21 +69,40 @@ __device__ __forceinline__ uint32_t scale_f16x2(uint32_t v, float f) {
     return (uint32_t)__half_as_ushort(__float2half_rn(x)) | ((uint32_t)__half_as_ushort(__float2half_rn(y)) << 16);
 }
 
-// Multiplies the staged coefficients [0, slots) of row m by f (a power of two): a row whose
-// coefficients outgrow the range its scale was chosen for.
-__device__ __noinline__ void rescale_row(const ProjEntry &e, int64_t m, int slots, float f) {
-    for (int h = 0; h < 2; ++h) {
-        uint4 *out = reinterpret_cast<uint4 *>(h ? e.A_lo : e.A_hi);
-        for (int ch = 0; ch < slots / 4; ++ch) {
-            uint4 *q = out + ((size_t)(ch >> 3) * e.M_pad + m) * 8 + ((ch & 7) ^ (int)(m & 7));
-            uint4 v = *q;
-            v.x = scale_f16x2(v.x, f);
-            v.y = scale_f16x2(v.y, f);
-            v.z = scale_f16x2(v.z, f);
-            v.w = scale_f16x2(v.w, f);
-            *q = v;
+// Multiplies the staged coefficients [0, slots) of this lane's row by f (a power of two; 1: left alone):
+// rows whose coefficients outgrow the range their scale was chosen for.  All lanes of the warp call it and
+// share each row's chunks, whole 128-byte lines at a time (one lane to a row walks its chunks one after
+// another, and rows outgrow their scales at different blocks, so the lanes of a warp wait for one another).
+__device__ __noinline__ void rescale_rows(const ProjEntry &e, int64_t m, int slots, float f) {
+    const int lane = threadIdx.x & 31;
+    for (unsigned todo = __ballot_sync(0xffffffffu, f != 1.f); todo; todo &= todo - 1) {
+        const int r = __ffs(todo) - 1;
+        const float g = __shfl_sync(0xffffffffu, f, r);
+        const int64_t row = m - lane + r;
+        for (int h = 0; h < 2; ++h) {
+            uint4 *out = reinterpret_cast<uint4 *>(h ? e.A_lo : e.A_hi);
+            for (int ch = lane; ch < slots / 4; ch += 32) {
+                uint4 *q = out + ((size_t)(ch >> 3) * e.M_pad + row) * 8 + ((ch & 7) ^ (int)(row & 7));
+                uint4 v = *q;
+                v.x = scale_f16x2(v.x, g);
+                v.y = scale_f16x2(v.y, g);
+                v.z = scale_f16x2(v.z, g);
+                v.w = scale_f16x2(v.w, g);
+                *q = v;
+            }
         }
     }
+}
+
+// Exponent of the scale of a row whose first nonzero block has largest component zmax, where the window
+// grows by 2^growth from that block to its largest in the ring: the ring's largest coefficient to about
+// 2^6, so that it may outgrow the window 500-fold before the row is rescaled (the range ends at 2^15), but the
+// block itself no lower than 2^-4, 20 bits above the smallest fp16 step.  Scales from the first block alone
+// had nearly every row rescaled under Blackman-Harris, which grows by more than 2^14: a segment of 16 200 rows x
+// 6681 frames took 5.89 ms and takes 1.00 (plain frames 1.20), the scan of 2^20 rows x 2048 frames 15.1 and 9.96.
+__device__ __forceinline__ float row_scale_for(float zmax, int growth) {
+    const int x = max(6 - growth, -4) - ilogbf(zmax);
+    return exp2f((float)max(-120, min(120, x)));
 }
 
 // Shared memory of a CTA of four warps: the basis, then per warp ring, modulation, transposition tile.
@@ -108,9 +127,8 @@ struct ProjSmem {
 // a block need (a tone sits in two or three of them, so their roundings average over fewer terms
 // than those of its B frames: bf16 pieces of them measured 1.4e-6 of the intensities on the scan of
 // 2048 frames, bf16 pieces of the frames 0.5e-6); the fp16 range is met by a power-of-two scale per
-// row, taken from the ring's first nonzero block (its largest component to [1, 2), 2^15 below the
-// range's end) and undone in the contraction's epilogue.  A row that outgrows it has its staged
-// coefficients rescaled.
+// row, taken from the ring's first nonzero block and the window (row_scale_for) and undone in the
+// contraction's epilogue.  A row that outgrows it has its staged coefficients rescaled.
 // CHECK: frame components beyond 65504 / e.f16_scale set DEVERR_FP16_RANGE (split-FP16 plans).
 // ONE: a launch of one entry, whose fields then are constants of the launch and not loads by index.
 template <int B, int R, bool SPLIT, bool CHECK, bool ONE>
@@ -318,9 +336,10 @@ __global__ void __launch_bounds__(128, ProjSmem<B, R, SPLIT>::kCtas)
                 float zmax = 0.f;
 #pragma unroll
                 for (int q = 0; q < R; ++q) zmax = fmaxf(zmax, fmaxf(fabsf(z(q).x), fabsf(z(q).y)));
-                if ((sc == 0.f ? zmax > 0.f : zmax * sc > 32768.f) && zmax < CUDART_INF_F) {
-                    const float ns = exp2f((float)-max(-120, min(120, ilogbf(zmax))));
-                    if (sc != 0.f) rescale_row(e, m, slot, ns / sc);
+                const bool fresh = (sc == 0.f ? zmax > 0.f : zmax * sc > 32768.f) && zmax < CUDART_INF_F;
+                if (__any_sync(0xffffffffu, fresh)) {
+                    const float ns = fresh ? row_scale_for(zmax, e.growth[k]) : sc;
+                    rescale_rows(e, m, slot, fresh && sc != 0.f ? ns / sc : 1.f);
                     sc = ns;
                 }
                 const float s = sc == 0.f ? 1.f : sc;

@@ -238,6 +238,27 @@ __global__ void band_mod_kernel(TableArgs a, int B, double fc, int n, float2 *mo
     mod[t] = v;
 }
 
+// One CTA per ring of `per` blocks (n in all): exponents of the blocks' largest |mod|, then of the ring's over them.
+__global__ void band_growth_kernel(int B, int per, int n, int total, const float2 *mod, unsigned char *growth) {
+    constexpr int kZero = -1000;                      // a block of zeros
+    __shared__ int top;
+    const int b0 = blockIdx.x * per, b1 = min(b0 + per, n);
+    auto exponent = [&](int blk) {
+        float w = 0.f;
+        for (int u = 0; u < B && blk * B + u < total; ++u)
+            w = fmaxf(w, fmaxf(fabsf(mod[blk * B + u].x), fabsf(mod[blk * B + u].y)));
+        return w > 0.f ? ilogbf(w) : kZero;
+    };
+    if (threadIdx.x == 0) top = kZero;
+    __syncthreads();
+    for (int blk = b0 + (int)threadIdx.x; blk < b1; blk += blockDim.x) atomicMax(&top, exponent(blk));
+    __syncthreads();
+    for (int blk = b0 + (int)threadIdx.x; blk < b1; blk += blockDim.x) {
+        const int x = exponent(blk);
+        growth[blk] = (unsigned char)(x == kZero ? 0 : min(top - x, 255));
+    }
+}
+
 // one thread per (energy, basis vector); a.cj holds c_j for FFT grids too
 __global__ void band_response_kernel(TableArgs a, BandTableArgs b, double *q_resp) {
     const int j = blockIdx.x * blockDim.x + threadIdx.x, q = blockIdx.y;
@@ -356,6 +377,13 @@ cudaError_t launch_band_merge(const BandMergeArgs &m, __nv_bfloat16 *T_hi, __nv_
 cudaError_t launch_band_mod(const TableArgs &t, const BandTableArgs &b, float2 *mod, cudaStream_t st) {
     const int n = (t.T + b.B - 1) / b.B * b.B;
     band_mod_kernel<<<(n + 127) / 128, 128, 0, st>>>(t, b.B, b.fc, n, mod);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_band_growth(const TableArgs &t, const BandTableArgs &b, const float2 *mod, unsigned char *growth,
+                               cudaStream_t st) {
+    const int n = (t.T + b.B - 1) / b.B;
+    band_growth_kernel<<<b.rounds, 256, 0, st>>>(b.B, b.rounds > 1 ? b.ring / b.B : n, n, n * b.B, mod, growth);
     return cudaGetLastError();
 }
 

@@ -1046,6 +1046,7 @@ ProjEntry proj_entry(const tacaw_plan_s *p, const Stream &s, const FrameGeom &g,
     e.A_lo = s.A_lo;
     e.A32 = s.A32;
     e.row_scale = s.row_scale();
+    e.growth = b.growth + (s.stage_start / b.B + blk0);
     if (p->f16) {
         e.f16_scale = p->f16_scale;
         e.err = p->d_err;

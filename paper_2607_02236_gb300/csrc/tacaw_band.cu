@@ -304,7 +304,8 @@ tacaw_status build_band_forms(tacaw_plan_s *p, Stream &s, int64_t room_bytes, Ba
         const size_t tp = (size_t)round_up(s.T, B), n1 = (size_t)b.wt1 * b.n_wt1;
         const size_t tw = rows * s.Nw_pad * 8;   // bytes of B_hi, of B_lo, or of B32
         const size_t t1 = b.S ? (size_t)b.S / B * R * n1 * 8 : 0;   // of T_hi, of T_lo
-        const size_t bytes = (split ? 2 : 1) * tw + 2 * t1 + ((size_t)K * s.Nw + n + tp + w.size() + centre.size() + s.Nw) * 8;
+        const size_t bytes = (split ? 2 : 1) * tw + 2 * t1 +
+                             ((size_t)K * s.Nw + n + tp + w.size() + centre.size() + s.Nw) * 8 + tp / B;
         if ((int64_t)bytes > room_bytes) continue;
         unsigned char *mem = nullptr;
         if (!dev_alloc(p, &mem, bytes)) break;   // no memory for this form's tables: frames, or the form built before
@@ -325,11 +326,13 @@ tacaw_status build_band_forms(tacaw_plan_s *p, Stream &s, int64_t room_bytes, Ba
         double *d_basis = d_resp + (size_t)K * s.Nw;
         b.mod = reinterpret_cast<float2 *>(d_basis + n);
         double *d_w = reinterpret_cast<double *>(b.mod + tp), *d_centre = d_w + w.size(), *d_cj = d_centre + centre.size();
+        b.growth = reinterpret_cast<unsigned char *>(d_cj + s.Nw);
         b.basis.assign(basis.begin(), basis.end());
         CU_CHECK(p, cudaMemcpy(d_basis, basis.data(), sizeof(double) * n, cudaMemcpyHostToDevice), "basis");
         ba.basis = d_basis;
         const TableArgs ta = stream_table_args(s, p->bf);
         CU_CHECK(p, launch_band_mod(ta, ba, b.mod, st), "band modulation");
+        if (split) CU_CHECK(p, launch_band_growth(ta, ba, b.mod, b.growth, st), "band window growth");
         if (b.S) {
             // first level, then the tiles' twiddles as those of blocks of S frames about each tile's centre
             std::vector<double> cj(s.Nw);

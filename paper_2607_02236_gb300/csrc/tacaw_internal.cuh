@@ -290,6 +290,10 @@ struct BandTableArgs {
     int rounds;                // flushes a segment
 };
 cudaError_t launch_band_mod(const TableArgs &t, const BandTableArgs &b, float2 *mod, cudaStream_t st);
+// growth [T / B rounded up]: exponent of the ratio of the window's largest value in the block's ring to its
+// largest in the block (0 for a block of zeros, at most 255), from mod
+cudaError_t launch_band_growth(const TableArgs &t, const BandTableArgs &b, const float2 *mod, unsigned char *growth,
+                               cudaStream_t st);
 // q_resp [R][Nw]: response of each basis vector at each energy (FP64; imaginary for the odd ones)
 cudaError_t launch_band_response(const TableArgs &t, const BandTableArgs &b, double *q_resp, cudaStream_t st);
 // split twiddles [rounds * slots / 32][2 Nw_pad][64] (pre-swizzled) or FP32 [rounds * slots][Nw_pad]
@@ -345,6 +349,8 @@ struct ProjEntry {
     __nv_bfloat16 *A_hi, *A_lo;   // split staging (fp16 pieces), or
     float2 *A32;                  // FP32 staging
     float *row_scale;          // split staging: [M_pad] scale of the row's staged coefficients (0: all zero so far)
+    const unsigned char *growth;   // split staging: exponent of the window's growth from each completed block
+                                   // to its largest in the ring
     float f16_scale;           // split-FP16 plans: frames are checked against the fp16 range at this
     uint32_t *err;             // scale (err not null)
     int64_t group_begin;       // set by the launcher: first of its groups of 128 rows

@@ -24,6 +24,7 @@ struct BandForm {
     int slots = 0;             // table rows per flush; the carry, then the row scales, follow
                                // the ring's first `slots` slots
     float2 *mod = nullptr;     // [T rounded up to B]
+    unsigned char *growth = nullptr;   // [blocks of T] (split path)
     std::vector<float> basis;  // [B/2][R]
     __nv_bfloat16 *B_hi = nullptr, *B_lo = nullptr;   // twiddles (split path)
     float2 *B32 = nullptr;                            // twiddles (FP32 path)

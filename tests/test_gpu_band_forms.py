@@ -201,3 +201,59 @@ def test_checkpoint_versions():
             plan.restore_state(state)
             push_all(plan, fr, [32], 96)
             assert np.array_equal(finish(plan)[0], want)
+
+
+def row_scales(plan):
+    """Scales of the rows' staged coefficients (the last section of a checkpoint between blocks)."""
+    return plan.save_state()[-4 * (-(-ROWS // 128) * 128):].copy().view(np.float32)
+
+
+@pytest.mark.parametrize("precision", ["split_bf16", "split_fp16"])
+def test_windows_that_start_low_keep_their_rows_scale(precision):
+    """Blackman-Harris grows by 2^14 from a segment's first block to its middle: the rows' scales, set with the
+    first block, take that into account and hold to the end."""
+    from paper_2607_02236_gb300 import TacawPlan
+    cfg = config(2048, 400, 120.0, window="blackmanharris")
+    fr = waves(2048, 13)
+    with TacawPlan([cfg], precision=precision) as plan:
+        push_all(plan, fr, [64], 0, 64)
+        assert ring_form(plan) == 64
+        first = row_scales(plan)
+        push_all(plan, fr, [64], 64)
+        assert np.array_equal(row_scales(plan), first)
+        I, Psi = finish(plan, psi=True)
+    assert_exact(I, fr, cfg, Psi)
+
+
+@pytest.mark.parametrize("precision,T,sizes,ring", [("split_bf16", 1024, [64], 64), ("split_fp16", 1024, [64], 64),
+                                                    ("split_bf16", 2048, [32], 32), ("split_bf16", 1024, [48], 64)])
+def test_rows_that_outgrow_their_scale(precision, T, sizes, ring):
+    """Bursts of 2^12 to 2^24 times the earlier signal, in a third of the rows and at places that differ from row
+    to row, have the staged coefficients of those rows rescaled, some of them twice."""
+    import torch
+    from paper_2607_02236_gb300 import TacawPlan
+    cfg = config(T, 1000 if ring == 64 else 400, 150.0 if ring == 64 else 120.0, window="rect")
+    fr = waves(T, 14, elastic=0.0) * 1e-4
+    g = torch.Generator(device="cuda").manual_seed(15)
+    row = torch.arange(ROWS, device="cuda")
+    for factor, a, b in ((2.0 ** 12, T // 8, T // 2), (2.0 ** 12, T // 2, 7 * T // 8)):
+        at_row = torch.randint(a, b, (ROWS,), device="cuda", generator=g)
+        at_row = torch.where(row % 3 == 1, at_row, T)
+        fr *= torch.where(torch.arange(T, device="cuda")[:, None] >= at_row[None, :], factor, 1.0)
+    with TacawPlan([cfg], precision=precision, **({"fp16_scale": 16.0} if precision == "split_fp16" else {})) as plan:
+        push_all(plan, fr, sizes, 0, sizes[0])
+        first = None
+        if sizes[0] == ring:
+            assert ring_form(plan) == ring
+            first = row_scales(plan)
+        push_all(plan, fr, sizes, sizes[0])
+        if first is not None:
+            changed = (row_scales(plan) != first)[:ROWS]
+            assert changed[1::3].all() and not changed[0::3].any()
+        I, Psi = finish(plan, psi=True)
+    # rows of very different size: each against its own peak
+    kw = dict(window_kind="rect", E_meV=cfg.E_meV)
+    psi, want = oracle.forward_pixels(fr[:, PIX].cpu().numpy(), **kw)
+    for k, p in enumerate(PIX):
+        assert rel_err_peak(I[:, p], want[:, k]) <= TOL, (p, p % 3)
+        assert rel_err_peak(Psi[:, p], psi[:, k]) <= TOL, (p, p % 3)
