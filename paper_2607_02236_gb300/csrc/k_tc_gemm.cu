@@ -810,6 +810,9 @@ __global__ void __maxnreg__(168) flush_tc_drain2_kernel(const __grid_constant__ 
             // then wait on nothing); compensated and FP64 accumulators are added at the end
             const int kind0 = epi_kind(a.e);
             const bool preload = (kind0 == EPI_ADD_KAHAN || kind0 == EPI_FINAL_KAHAN) && a.e.acc_c == nullptr;
+            // a row of coefficients scaled so far up (a ring in the window's far tail) that its accumulators would
+            // overflow at that scale: they are added behind the products instead, read once more
+            bool late = false;
             {
                 // this thread's energies j0 .. j0 + nv - 1 of row mrow (accumulators [Nw_pad][M_pad])
                 const int64_t mrow = (int64_t)m0 + q4 * 32 + lane;
@@ -831,8 +834,12 @@ __global__ void __maxnreg__(168) flush_tc_drain2_kernel(const __grid_constant__ 
                 }
                 if (BAND && preload && a.row_scale) {
                     const float ps = 1.f / row_factor(a, mrow);
+                    float top = 0.f;
 #pragma unroll
-                    for (int i = 0; i < kDrainCols; ++i) sum[i] *= ps;
+                    for (int i = 0; i < kDrainCols; ++i) top = fmaxf(top, fabsf(sum[i]));
+                    late = !(top * ps < 8e37f);
+#pragma unroll
+                    for (int i = 0; i < kDrainCols; ++i) sum[i] = late ? 0.f : sum[i] * ps;
                 }
             }
             for (int lc = 0; lc + 1 < n_chunks; ++lc, ++hc) {
@@ -872,6 +879,17 @@ __global__ void __maxnreg__(168) flush_tc_drain2_kernel(const __grid_constant__ 
                 const float rf = row_factor(a, row.m);
 #pragma unroll
                 for (int i = 0; i < kDrainCols; ++i) sum[i] *= rf;
+                if (late) {
+                    const int j0 = jbase + (col0 >> 1), nv = row.valid ? max(0, min(cols >> 1, a.e.Nw - j0)) : 0;
+                    const float2 *ap = a.e.acc_s + (size_t)j0 * (size_t)a.e.M_pad + (size_t)row.m;
+#pragma unroll
+                    for (int i = 0; i < kDrainCols / 2; ++i) {
+                        const float2 v = i < nv ? *ap : make_float2(0.f, 0.f);
+                        ap += a.e.M_pad;
+                        sum[2 * i] += v.x;
+                        sum[2 * i + 1] += v.y;
+                    }
+                }
             }
             // with preloaded sums an update of the accumulators is a store, a finalize one without
             // earlier flushes

@@ -257,3 +257,20 @@ def test_rows_that_outgrow_their_scale(precision, T, sizes, ring):
     for k, p in enumerate(PIX):
         assert rel_err_peak(I[:, p], want[:, k]) <= TOL, (p, p % 3)
         assert rel_err_peak(Psi[:, p], psi[:, k]) <= TOL, (p, p % 3)
+
+
+@pytest.mark.parametrize("precision", ["split_bf16", "split_fp16"])
+def test_accumulators_of_rings_in_a_far_tail(precision):
+    """Four flushes under a Gauss window whose first and last rings hold 1e-38 of its maximum: their rows are
+    scaled up by as much as 2^120, where the plain FP32 accumulators of the rings before have no place."""
+    from paper_2607_02236_gb300 import TacawPlan
+    cfg = config(2048, 1000, 150.0, window="gauss", window_param=38.8)
+    fr = waves(2048, 17) * 1e3
+    with TacawPlan([cfg], precision=precision, k_stage=512, accum="fp32",
+                   **({"fp16_scale": 4.0} if precision == "split_fp16" else {})) as plan:
+        push_all(plan, fr, [64], 0, 1600)
+        assert ring_form(plan) == 64
+        push_all(plan, fr, [64], 1600)
+        I, Psi = finish(plan, psi=True)
+        assert plan.info()["flushes"] == 4
+    assert_exact(I, fr, cfg, Psi)
