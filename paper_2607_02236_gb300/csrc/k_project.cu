@@ -55,6 +55,25 @@ __device__ __forceinline__ void proj_copy(float2 *dst, const float2 *src, int by
                  : "memory");
 }
 
+// tot + rest += part, the rounding of tot kept in rest (Knuth's two-sum).  The residual sums behind the exact
+// mean run in FP32 over a few frames only, as in the conversions of plain frames (up to 32 on the split path, 8
+// on the FP32 path), and are exact from there on.  On the FP32 path a block has up to 16 such partial sums: FP64
+// adds would be two additions and two conversions each, on a pipe with a 64th of the FP32 rate; this costs the
+// FP32 scan (blocks of 128 frames, R 36) 6.10 ms instead of 6.05.
+__device__ __forceinline__ void add_partial(float2 &tot, float2 &rest, float2 part) {
+    const float2 t = __fadd2_rn(tot, part);
+    const float2 b = __fadd2_rn(t, make_float2(-tot.x, -tot.y));       // the part as it went in
+    const float2 a = __fadd2_rn(t, make_float2(-b.x, -b.y));           // tot as it went in
+    rest = __fadd2_rn(rest, __fadd2_rn(__fadd2_rn(tot, make_float2(-a.x, -a.y)),
+                                       __fadd2_rn(part, make_float2(-b.x, -b.y))));
+    tot = t;
+}
+// (one lane alone adds to a row in a launch: the sum's order is fixed)
+__device__ __forceinline__ void add_residual(double2 *sum_res, float2 tot, float2 rest) {
+    atomicAdd(&sum_res->x, (double)tot.x + (double)rest.x);
+    atomicAdd(&sum_res->y, (double)tot.y + (double)rest.y);
+}
+
 // (re, im) of a scaled coefficient as fp16 hi + lo (22 bits), re in the low half.
 __device__ __forceinline__ void proj_split_f16(float2 r, uint32_t &hi, uint32_t &lo) {
     const __half2 h = __float22half2_rn(r);
@@ -247,7 +266,9 @@ __global__ void __launch_bounds__(128, ProjSmem<B, R, SPLIT>::kCtas)
             }
             const bool whole = f0 >= 0 && f0 + B <= e.n;
             // coefficient pairs (2 i, 2 i + 1) of the even and the odd half
-            float2 er[RP], ei[RP], dr[RP], di[RP], sum = make_float2(0.f, 0.f);
+            float2 er[RP], ei[RP], dr[RP], di[RP];
+            // sums of the residuals: SPLIT: tot of the block's first half, sum of its second; else add_partial's
+            float2 sum = make_float2(0.f, 0.f), tot = sum, rest = sum;
 #pragma unroll
             for (int i = 0; i < RP; ++i) er[i] = ei[i] = dr[i] = di[i] = make_float2(0.f, 0.f);
 #pragma unroll 1
@@ -263,7 +284,7 @@ __global__ void __launch_bounds__(128, ProjSmem<B, R, SPLIT>::kCtas)
 #pragma unroll
                     for (int i = 0; i < 2 * KP; ++i) {
                         y[i] = __fadd2_rn(y[i], nmu);
-                        sum = __fadd2_rn(sum, y[i]);
+                        (SPLIT && i < KP ? tot : sum) = __fadd2_rn(SPLIT && i < KP ? tot : sum, y[i]);
                     }
                 } else {
 #pragma unroll
@@ -271,9 +292,13 @@ __global__ void __launch_bounds__(128, ProjSmem<B, R, SPLIT>::kCtas)
                         const int f = f0 + (i < KP ? KP * st + i : B - 1 - KP * st - (i - KP));
                         if (f >= 0 && f < e.n) {   // (carried frames are residuals, already counted)
                             y[i] = __fadd2_rn(y[i], nmu);
-                            sum = __fadd2_rn(sum, y[i]);
+                            (SPLIT && i < KP ? tot : sum) = __fadd2_rn(SPLIT && i < KP ? tot : sum, y[i]);
                         }
                     }
+                }
+                if (!SPLIT) {                     // (eight frames a stage)
+                    add_partial(tot, rest, sum);
+                    sum = make_float2(0.f, 0.f);
                 }
                 if (CHECK) {
 #pragma unroll
@@ -320,11 +345,7 @@ __global__ void __launch_bounds__(128, ProjSmem<B, R, SPLIT>::kCtas)
                     }
                 }
             }
-            // (this lane alone adds to its row in the launch: the sum's order is fixed)
-            if ((int64_t)m < e.g.M) {
-                atomicAdd(&e.sum_res[m].x, (double)sum.x);
-                atomicAdd(&e.sum_res[m].y, (double)sum.y);
-            }
+            if ((int64_t)m < e.g.M) add_residual(&e.sum_res[m], tot, SPLIT ? sum : rest);
             // coefficient q of the block: even half first
             auto z = [&](int q) {
                 const int i = (q % RH) >> 1;
@@ -391,7 +412,6 @@ __global__ void __launch_bounds__(128, ProjSmem<B, R, SPLIT>::kCtas)
             const bool valid = (int64_t)m < e.g.M;
             const float2 *src = e.g.base + (valid ? proj_row(e.g, m) : 0);
             float2 *carry = e.carry + m;
-            float br = 0.f, bi = 0.f;
             const int base = e.nblk > 0 ? -done : e.c0;   // carry slot of pushed frame f: base + f
 #pragma unroll 1
             for (int f = first; f < e.n; f += 8) {
@@ -399,19 +419,16 @@ __global__ void __launch_bounds__(128, ProjSmem<B, R, SPLIT>::kCtas)
 #pragma unroll
                 for (int i = 0; i < 8; ++i)
                     v[i] = valid && f + i < e.n ? __ldcs(src + (int64_t)(f + i) * e.g.pitch_frame) : mu;
+                float2 sum = make_float2(0.f, 0.f);
 #pragma unroll
                 for (int i = 0; i < 8; ++i)
                     if (f + i < e.n) {
                         const float2 y = make_float2(v[i].x - mu.x, v[i].y - mu.y);
-                        br += y.x;
-                        bi += y.y;
+                        sum = __fadd2_rn(sum, y);
                         if (CHECK) amax = fmaxf(amax, fmaxf(fabsf(y.x), fabsf(y.y)));
                         carry[(int64_t)(base + f + i) * e.M_pad] = y;
                     }
-            }
-            if (valid) {
-                atomicAdd(&e.sum_res[m].x, (double)br);
-                atomicAdd(&e.sum_res[m].y, (double)bi);
+                if (valid) add_residual(&e.sum_res[m], sum, make_float2(0.f, 0.f));
             }
         }
         if (CHECK && amax * e.f16_scale > 65504.f) atomicOr(e.err, DEVERR_FP16_RANGE);
@@ -432,23 +449,25 @@ __global__ void __launch_bounds__(128) carry_group_kernel(const __grid_constant_
     const float2 *src = e.g.base + proj_row(e.g, m);
     float2 *carry = e.carry + m + (int64_t)e.c0 * e.M_pad;
     const float2 mu = e.mu_hat[m];
-    float br = 0.f, bi = 0.f, amax = 0.f;
+    float2 tot = make_float2(0.f, 0.f), rest = tot;
+    float amax = 0.f;
     for (int f0 = 0; f0 < e.n; f0 += 16) {
         float2 v[16];
 #pragma unroll
         for (int f = 0; f < 16; ++f) v[f] = f0 + f < e.n ? __ldcs(src + (int64_t)(f0 + f) * pitch) : mu;
+        float2 sum[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};   // of eight frames each
 #pragma unroll
         for (int f = 0; f < 16; ++f)
             if (f0 + f < e.n) {
                 const float2 y = make_float2(v[f].x - mu.x, v[f].y - mu.y);
-                br += y.x;
-                bi += y.y;
+                sum[f / 8] = __fadd2_rn(sum[f / 8], y);
                 if (CHECK) amax = fmaxf(amax, fmaxf(fabsf(y.x), fabsf(y.y)));
                 carry[(int64_t)(f0 + f) * e.M_pad] = y;
             }
+        add_partial(tot, rest, sum[0]);
+        add_partial(tot, rest, sum[1]);
     }
-    atomicAdd(&e.sum_res[m].x, (double)br);
-    atomicAdd(&e.sum_res[m].y, (double)bi);
+    add_residual(&e.sum_res[m], tot, rest);
     if (CHECK && amax * e.f16_scale > 65504.f) atomicOr(e.err, DEVERR_FP16_RANGE);
 }
 

@@ -274,3 +274,27 @@ def test_accumulators_of_rings_in_a_far_tail(precision):
         I, Psi = finish(plan, psi=True)
         assert plan.info()["flushes"] == 4
     assert_exact(I, fr, cfg, Psi)
+
+
+@pytest.mark.parametrize("precision,ring,sizes", [("fp32", 128, [128]), ("fp32", 128, [200, 56]), ("fp32", 128, [16]),
+                                                  ("split_bf16", 64, [64]), ("split_bf16", 64, [16]),
+                                                  ("split_fp16", 64, [100, 28])])
+def test_residual_sums_are_exact_to_a_few_frames(precision, ring, sizes):
+    """The sums behind the exact mean run in FP32 over 8 frames (FP32 path) or 32 (split path) and are exact from
+    there on: frames of 1 + 2^-20 (2^-19) sum without a rounding up to 8 (32) of them, and lose bits in longer
+    FP32 sums.  The first 32 frames, which give the provisional mean, are zero."""
+    from paper_2607_02236_gb300 import TacawPlan
+    T = 1024
+    cfg = config(T, 1000, 150.0)
+    fr = waves(T, 11, elastic=0.0) * 0
+    one = 1 + 2.0 ** (-20 if precision == "fp32" else -19)
+    fr[32:] = one * (1 - 1j)
+    with TacawPlan([cfg], precision=precision) as plan:
+        push_all(plan, fr, [32] if sizes == [16] else sizes, 0, 32 if sizes == [16] else sizes[0])
+        a = 32 if sizes == [16] else sizes[0]
+        push_all(plan, fr, sizes, a, 768)
+        assert ring_form(plan) == ring
+        state = plan.save_state()
+    off = 48 + 48 + 8 + 8 * ROWS           # behind the header, the counters and the provisional means
+    sums = state[off:off + 16 * ROWS].copy().view(np.complex128)
+    assert np.all(sums == (768 - 32) * one * (1 - 1j))
