@@ -148,7 +148,8 @@ struct ProjSmem {
 // 2048 frames, bf16 pieces of the frames 0.5e-6); the fp16 range is met by a power-of-two scale per
 // row, taken from the ring's first nonzero block and the window (row_scale_for) and undone in the
 // contraction's epilogue.  A row that outgrows it has its staged coefficients rescaled.
-// CHECK: frame components beyond 65504 / e.f16_scale set DEVERR_FP16_RANGE (split-FP16 plans).
+// CHECK: frame components beyond 65504 / e.f16_scale set DEVERR_FP16_RANGE (split-FP16 plans): of the frames less
+// their provisional mean, as those of plain frames, or with e.check_raw as they are (a kept mean stays in plain frames).
 // ONE: a launch of one entry, whose fields then are constants of the launch and not loads by index.
 template <int B, int R, bool SPLIT, bool CHECK, bool ONE>
 __global__ void __launch_bounds__(128, ProjSmem<B, R, SPLIT>::kCtas)
@@ -280,6 +281,13 @@ __global__ void __launch_bounds__(128, ProjSmem<B, R, SPLIT>::kCtas)
                 get = (get + 1) % NS;
                 copy_stage();                     // into the slot read one stage ago
                 const float2 nmu = make_float2(-mu.x, -mu.y);
+                if (CHECK && e.check_raw) {       // (carried frames were checked when they came)
+#pragma unroll
+                    for (int i = 0; i < 2 * KP; ++i) {
+                        const int f = f0 + (i < KP ? KP * st + i : B - 1 - KP * st - (i - KP));
+                        if (f >= 0) amax = fmaxf(amax, fmaxf(fabsf(y[i].x), fabsf(y[i].y)));
+                    }
+                }
                 if (whole) {
 #pragma unroll
                     for (int i = 0; i < 2 * KP; ++i) {
@@ -300,7 +308,7 @@ __global__ void __launch_bounds__(128, ProjSmem<B, R, SPLIT>::kCtas)
                     add_partial(tot, rest, sum);
                     sum = make_float2(0.f, 0.f);
                 }
-                if (CHECK) {
+                if (CHECK && !e.check_raw) {
 #pragma unroll
                     for (int i = 0; i < 2 * KP; ++i) amax = fmaxf(amax, fmaxf(fabsf(y[i].x), fabsf(y[i].y)));
                 }
@@ -425,7 +433,10 @@ __global__ void __launch_bounds__(128, ProjSmem<B, R, SPLIT>::kCtas)
                     if (f + i < e.n) {
                         const float2 y = make_float2(v[i].x - mu.x, v[i].y - mu.y);
                         sum = __fadd2_rn(sum, y);
-                        if (CHECK) amax = fmaxf(amax, fmaxf(fabsf(y.x), fabsf(y.y)));
+                        if (CHECK) {
+                            const float2 c = e.check_raw ? v[i] : y;
+                            amax = fmaxf(amax, fmaxf(fabsf(c.x), fabsf(c.y)));
+                        }
                         carry[(int64_t)(base + f + i) * e.M_pad] = y;
                     }
                 if (valid) add_residual(&e.sum_res[m], sum, make_float2(0.f, 0.f));
@@ -461,7 +472,10 @@ __global__ void __launch_bounds__(128) carry_group_kernel(const __grid_constant_
             if (f0 + f < e.n) {
                 const float2 y = make_float2(v[f].x - mu.x, v[f].y - mu.y);
                 sum[f / 8] = __fadd2_rn(sum[f / 8], y);
-                if (CHECK) amax = fmaxf(amax, fmaxf(fabsf(y.x), fabsf(y.y)));
+                if (CHECK) {
+                    const float2 c = e.check_raw ? v[f] : y;
+                    amax = fmaxf(amax, fmaxf(fabsf(c.x), fabsf(c.y)));
+                }
                 carry[(int64_t)(f0 + f) * e.M_pad] = y;
             }
         add_partial(tot, rest, sum[0]);

@@ -1023,6 +1023,16 @@ tacaw_status push_counted(tacaw_plan_s *p, UserStream &u, int n, cudaStream_t st
     return TACAW_OK;
 }
 
+// A ring's first push, of n frames: its form, and with a segment's first ring whether the provisional mean
+// leaves the frames.
+void start_ring(tacaw_plan_s *p, Stream &s, int n) {
+    // split FP16 with a kept mean: plain frames hold the mean (their residuals could leave the fp16 range that the
+    // frames themselves are held to), coefficients do not, so a segment keeps to the kind its first ring has
+    const bool one_kind = p->f16 && s.shift_mean && s.pushed > 0;
+    s.form = one_kind && !s.shifted ? -1 : choose_form(p, s, n, one_kind);
+    if (s.pushed == 0) s.shifted = s.shift_mean && (!p->f16 || s.form >= 0);
+}
+
 // The conversion of one push of n frames (inside the ring) on the ring's band-limited form.
 ProjEntry proj_entry(const tacaw_plan_s *p, const Stream &s, const FrameGeom &g, int n) {
     const BandForm &b = s.band[s.form];
@@ -1049,6 +1059,7 @@ ProjEntry proj_entry(const tacaw_plan_s *p, const Stream &s, const FrameGeom &g,
     e.growth = b.growth + (s.stage_start / b.B + blk0);
     if (p->f16) {
         e.f16_scale = p->f16_scale;
+        e.check_raw = !s.d.subtract_mean;
         e.err = p->d_err;
     }
     return e;
@@ -1062,11 +1073,11 @@ tacaw_status push_internal(tacaw_plan_s *p, Stream &s, const float2 *frames, int
         tacaw_status r = flush_due(p, st);
         if (r != TACAW_OK) return r;
     }
+    if (s.staged == 0) start_ring(p, s, std::min(n_frames, s.ring));
     if (s.pushed == 0 && s.removes_mean()) {
         CU_CHECK(p, launch_mean(g, n_frames, s.mu_hat, st), "provisional mean");
         p->launches++;
     }
-    if (s.staged == 0) s.form = choose_form(p, s, std::min(n_frames, s.ring));
     if (p->pipe && p->pend.active && s.form >= 0) {
         // band-limited forms are converted at push time (into the staging area the pending
         // contraction does not read); the pending contraction still goes out with the finalize
@@ -1084,7 +1095,7 @@ tacaw_status push_internal(tacaw_plan_s *p, Stream &s, const float2 *frames, int
     int done = 0;
     while (done < n_frames) {
         const int chunk = std::min(n_frames - done, s.ring - s.staged);
-        if (s.staged == 0) s.form = choose_form(p, s, chunk);
+        if (s.staged == 0) start_ring(p, s, chunk);
         FrameGeom gc = g;
         gc.base = g.base + (int64_t)done * g.pitch_frame;
         if (p->in_place) {
@@ -1618,7 +1629,7 @@ tacaw_status tacaw_push_frames_group(tacaw_plan_t p, int n, const int *stream_id
         const bool in_ring = u.N <= 1 && !p->in_place && !p->pipe && u.pushed >= u.skip && !s.due &&
                              s.staged + n_frames[i] <= s.ring;
         // the form is the ring's: its first push picks it, later ones continue it
-        if (in_ring && s.staged == 0) s.form = choose_form(p, s, n_frames[i]);
+        if (in_ring && s.staged == 0) start_ring(p, s, n_frames[i]);
         banded[i] = in_ring && s.form >= 0;
         if (banded[i]) continue;
         if (in_ring && split && convert_split_groupable(p->bf, s.staged, n_frames[i])) {

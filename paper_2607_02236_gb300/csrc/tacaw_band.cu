@@ -358,7 +358,7 @@ tacaw_status build_band_forms(tacaw_plan_s *p, Stream &s, int64_t room_bytes, Ba
         CU_CHECK(p, launch_band_response(ta, ba, d_resp, st), "band response");
         CU_CHECK(p, launch_band_twiddles(ta, ba, d_resp, b.B_hi, b.B_lo, b.B32, st), "band twiddles");
         s.band[s.n_band++] = b;
-        s.shift_mean = !s.d.subtract_mean && !p->f16;   // (split FP16 checks the range of the frames as they are)
+        s.shift_mean = !s.d.subtract_mean;
     }
     return TACAW_OK;
 }
@@ -370,10 +370,11 @@ tacaw_status build_band_forms(tacaw_plan_s *p, Stream &s, int64_t room_bytes, Ba
 // product, a tenth more on coefficients (shorter sums, drained more often).  Both sides at the line: six
 // partitions pushed 16 frames at a time, 300 energies: frames 14.9 + 20.1 ms, blocks of 32 with
 // half their frames carried 21.2 + 11.0 ms.
-int choose_form(const tacaw_plan_s *p, const Stream &s, int n) {
+int choose_form(const tacaw_plan_s *p, const Stream &s, int n, bool band_only) {
     const bool split = p->prec == TACAW_PREC_SPLIT_BF16;
     const double product = split ? 0.0139 : 0.142, push_rows = (double)s.M * n;
     double best = 0.97 * (2.65 + 8.0 / n + 3e6 / push_rows + (n % 4 ? 0.5 : 0.0) + product * s.Nw_pad);
+    if (band_only) best = HUGE_VAL;
     int form = -1;
     for (int i = 0; i < s.n_band; ++i) {
         const BandForm &b = s.band[i];

@@ -352,7 +352,8 @@ struct ProjEntry {
     const unsigned char *growth;   // split staging: exponent of the window's growth from each completed block
                                    // to its largest in the ring
     float f16_scale;           // split-FP16 plans: frames are checked against the fp16 range at this
-    uint32_t *err;             // scale (err not null)
+    uint32_t *err;             // scale (err not null), less their provisional mean, or with check_raw (a
+    int check_raw;             // stream that keeps its mean) as they are
     int64_t group_begin;       // set by the launcher: first of its groups of 128 rows
 };
 struct ProjGroup {

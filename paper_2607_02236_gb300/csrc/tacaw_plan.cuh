@@ -110,7 +110,8 @@ struct Stream {
     // with other forms).  Streams with band-limited forms: their coefficients' sums of an elastic line a
     // hundred times the signal were 2.0e-6 of the intensities off, the frames' 1.1e-6.
     bool shift_mean = false;
-    bool removes_mean() const { return d.subtract_mean || shift_mean; }
+    bool shifted = false;      // shift_mean, and this segment's frames are without it (start_ring)
+    bool removes_mean() const { return d.subtract_mean || shifted; }
     // staged slots of the ring: frames, or the coefficients of its blocks (whole ones, and at the
     // segment's end a short one)
     int ring_slots() const {
@@ -241,8 +242,8 @@ struct BandCache {
 // device memory; a stream without any keeps staging frames.  only: just the form with blocks of that many frames.
 tacaw_status build_band_forms(tacaw_plan_s *p, Stream &s, int64_t room_bytes, BandCache &cache, cudaStream_t st,
                               int only = 0);
-// The staging form a ring takes whose first push has n frames (-1: frames).
-int choose_form(const tacaw_plan_s *p, const Stream &s, int n);
+// The staging form a ring takes whose first push has n frames (-1: frames, unless band_only and s has a form).
+int choose_form(const tacaw_plan_s *p, const Stream &s, int n, bool band_only = false);
 // Table arguments of stream s after its tables were built.
 TableArgs stream_table_args(const Stream &s, int block_frames);
 

@@ -37,7 +37,7 @@ struct StateHeader {
 };
 struct StreamCounters {
     int64_t pushed, staged, stage_start, flushes, seg;
-    int32_t due;
+    int32_t due;              // bit 0: a full ring awaits its flush; bit 1: Stream::shifted
     int32_t form;             // staging form of the ring: 0 frames, else the block length B of its band-limited form
 };
 struct UserCounters {
@@ -173,7 +173,7 @@ std::vector<StreamCounters> plan_counters(const tacaw_plan_s *p) {
     std::vector<StreamCounters> c(p->s.size());
     for (size_t i = 0; i < p->s.size(); ++i) {
         const Stream &s = p->s[i];
-        c[i] = StreamCounters{s.pushed, s.staged, s.stage_start, s.flushes, s.seg, s.due ? 1 : 0,
+        c[i] = StreamCounters{s.pushed, s.staged, s.stage_start, s.flushes, s.seg, (s.due ? 1 : 0) | (s.shifted ? 2 : 0),
                               s.form >= 0 ? s.band[s.form].B : 0};
     }
     return c;
@@ -223,7 +223,7 @@ tacaw_status check_counters(const tacaw_plan_s *p, const std::vector<StreamCount
         const bool ok = k.pushed >= 0 && k.pushed <= s.T && k.staged >= 0 && k.staged <= s.ring &&
                         k.stage_start >= 0 && k.stage_start + k.staged == k.pushed && k.flushes >= 0 &&
                         k.flushes <= k.stage_start && (s.needs_acc || k.flushes == 0) &&
-                        (!p->in_place || k.staged == 0) && (k.due == 0 || (k.due == 1 && k.staged == s.ring)) &&
+                        (!p->in_place || k.staged == 0) && (k.due & ~3) == 0 && ((k.due & 1) == 0 || k.staged == s.ring) &&
                         (k.form == 0 || (k.staged > 0 && (k.form == 32 || k.form == 64 || k.form == 128))) &&
                         k.seg >= s.lane && (k.seg - s.lane) % u.lanes == 0 &&
                         k.seg < s.lane + (int64_t)u.lanes * (u.N + 1);
@@ -332,6 +332,12 @@ tacaw_status tacaw_restore_state(tacaw_plan_t p, const void *h_state, int64_t by
     // a ring in a form whose tables this plan had no room for at its creation: they are built now
     BandCache bases;
     for (size_t i = 0; i < p->s.size(); ++i) {
+        // (a split-FP16 segment without its kept mean goes on in coefficients)
+        if (p->f16 && (cnt[i].due & 2) && cnt[i].form == 0 && p->s[i].n_band == 0) {
+            c = build_band_forms(p, p->s[i], INT64_MAX, bases, st);
+            if (c != TACAW_OK) return c;
+            if (p->s[i].n_band == 0) return fail(TACAW_ERR_OOM, "checkpoint: no memory for stream %zu's band-limited forms", i);
+        }
         if (cnt[i].form == 0 || band_of(p->s[i], cnt[i].form) >= 0) continue;
         c = build_band_forms(p, p->s[i], INT64_MAX, bases, st, cnt[i].form);
         if (c != TACAW_OK) return c;
@@ -355,7 +361,8 @@ tacaw_status tacaw_restore_state(tacaw_plan_t p, const void *h_state, int64_t by
         s.flushes = (int)cnt[i].flushes;
         s.form = band_of(s, cnt[i].form);
         s.seg = cnt[i].seg;
-        s.due = cnt[i].due != 0;
+        s.due = cnt[i].due & 1;
+        s.shifted = (cnt[i].due & 2) != 0;
         s.due_stream = st;
         s.h_pushes.clear();
     }

@@ -298,3 +298,51 @@ def test_residual_sums_are_exact_to_a_few_frames(precision, ring, sizes):
     off = 48 + 48 + 8 + 8 * ROWS           # behind the header, the counters and the provisional means
     sums = state[off:off + 16 * ROWS].copy().view(np.complex128)
     assert np.all(sums == (768 - 32) * one * (1 - 1j))
+
+
+@pytest.mark.parametrize("nw,sizes,ring", [(400, [32], 32), (1000, [64], 64)])
+def test_split_fp16_kept_mean_outside_the_energies(nw, sizes, ring):
+    """A kept elastic line 300 times the signal, 20 meV below the energies: it is taken out of the frames before
+    they become coefficients, whose 22 bits would otherwise be spent on it."""
+    from paper_2607_02236_gb300 import TacawPlan
+    cfg = config(2048, nw, 100.0, window="rect", subtract_mean=False, E_meV=list(20.0 + np.arange(nw) * (100.0 / nw)))
+    fr = waves(2048, 19, elastic=30.0)
+    with TacawPlan([cfg], precision="split_fp16", fp16_scale=1024.0) as plan:
+        push_all(plan, fr, sizes, 0, 256)
+        assert ring_form(plan) == ring
+        push_all(plan, fr, sizes, 256)
+        I, Psi = finish(plan, psi=True)
+    assert_exact(I, fr, cfg, Psi)
+
+
+@pytest.mark.parametrize("first,ring", [(64, 64), (8, 0)])
+def test_split_fp16_kept_mean_range(first, ring):
+    """Frames that change sign after the first 32, at 0.94 of the fp16 range: accepted, with residuals beyond the
+    range, in a segment of two rings that both take the first one's kind of form.  Beyond the range: refused."""
+    from paper_2607_02236_gb300 import TacawError, TacawPlan
+    cfg = config(1024, 1000, 150.0, subtract_mean=False)
+    fr = waves(1024, 21, elastic=0.0) * 0.1
+    fr[:32] += 15 - 15j
+    fr[32:] -= 15 - 15j
+    with TacawPlan([cfg], precision="split_fp16", k_stage=512) as plan:
+        push_all(plan, fr, [first], 0, 512)
+        push_all(plan, fr, [8 if ring else 64], 512, 576)
+        assert (ring_form(plan) > 0) == (ring > 0)
+        state = plan.save_state()
+        push_all(plan, fr, [64], 576)
+        I, _ = finish(plan)
+        if ring:
+            assert_exact(I, fr, cfg)
+        plan.restore_state(state)
+        push_all(plan, fr, [64], 576)
+        assert np.array_equal(finish(plan)[0], I)
+        for t in (1, 500, 1000):
+            plan.reset()
+            bad = fr[t].clone()
+            fr[t, 7] = 16.1
+            with pytest.raises(TacawError, match="fp16 range"):
+                push_all(plan, fr, [first])
+                finish(plan)
+            fr[t] = bad
+            plan.close()
+            plan.__init__([cfg], precision="split_fp16", k_stage=512)
