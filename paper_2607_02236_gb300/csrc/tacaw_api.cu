@@ -1462,8 +1462,13 @@ tacaw_status tacaw_plan_create(const tacaw_plan_desc *desc, tacaw_plan_t *out) {
     BandCache bases;
     for (auto &s : p->s) room -= 12 * (int64_t)s.T_pad * s.Nw_pad;
     for (size_t i = 0; i < p->s.size() && rc == TACAW_OK; ++i) {
+        Stream &s = p->s[i];
+        if (s.lane > 0) {
+            share_band_forms(p->s[i - s.lane], s);   // the lanes of a Welch average have the same tables
+            continue;
+        }
         const int64_t before = p->bytes;
-        rc = build_band_forms(p, p->s[i], room, bases, st);
+        rc = build_band_forms(p, s, room, bases, st);
         room -= p->bytes - before;
     }
     for (auto &u : p->us) {

@@ -195,6 +195,39 @@ namespace {
 // Segments and rings shorter than this keep staging frames: their passes are bound by launches.
 constexpr int kBandMinT = 512;
 
+// Times a (row, frame), in picoseconds, of a ring whose pushes have n frames, staged as frames and as blocks of B
+// whose contraction costs `work` products: fitted to measurements (2^16 to 2^20 rows, 8 to 64 frames a push, 60
+// to 1000 energies).  A push of frames 2.65 + 8 / n and 3 us a launch (0.5 more where it parts the 16-byte
+// chunks of 4 frames); a push of whole blocks 2.3 + 8 / n and 4 us a launch, and 3.7 for the share of the frames
+// that passes through the carry; the contraction 0.0139 (split) or 0.142 (FP32) a product, a tenth more on
+// coefficients (shorter sums, drained more often).
+struct FormCost {
+    double product, rows;
+    int Nw_pad;
+    FormCost(const tacaw_plan_s *p, const Stream &s)
+        : product(p->prec == TACAW_PREC_SPLIT_BF16 ? 0.0139 : 0.142), rows((double)s.M), Nw_pad(s.Nw_pad) {}
+    double frames(int n) const {
+        return 0.97 * (2.65 + 8.0 / n + 3e6 / (rows * n) + (n % 4 ? 0.5 : 0.0) + product * Nw_pad);
+    }
+    double blocks(int n, int B, double work) const {
+        // share of the frames that wait in the carry, taking the ring's other pushes to be like its first:
+        // none for whole blocks, all but the completing push's for parts of a block, all for other sizes
+        // below a block (they drift against the blocks), a block's worth for longer ones
+        const double f = n % B == 0 ? 0.0 : B % n == 0 ? 1.0 - (double)n / B : n < B ? 1.0 : (double)B / n;
+        return 2.3 + 8.0 / std::max(n, 32) + 4e6 / (rows * n) + 3.7 * f + 1.1 * product * work;
+    }
+};
+
+// Whether the rule can pick blocks of B over frames for a push of some length (a ring's first push has up to
+// `most` frames).  Beyond two blocks both the launches' difference and the share carried fall with n, so the
+// lengths up to there, the longest whole number of blocks and the four longest (chunks parted or not) decide.
+bool ever_picked(const FormCost &c, int B, double work, int most) {
+    auto picks = [&](int n) { return n > 0 && n <= most && c.blocks(n, B, work) < c.frames(n); };
+    for (int n = 1; n <= 2 * B; ++n)
+        if (picks(n)) return true;
+    return picks(most / B * B) || picks(most) || picks(most - 1) || picks(most - 2) || picks(most - 3);
+}
+
 // Two-level contraction of a form's coefficients (split path): superblock length S and rank r an energy
 // tile, for the least complex products a (row, frame): R / B of the first level's columns, r / S of the
 // energies, and 200 a coefficient written and read (16 bytes at the copy rate against 0.0128 ps a
@@ -272,9 +305,14 @@ tacaw_status build_band_forms(tacaw_plan_s *p, Stream &s, int64_t room_bytes, Ba
     const double beta = (hi - lo) * dt_ps / kPlanck_meV_ps;
     if (!(beta < 0.5)) return TACAW_OK;   // no form pays (R / B near 1)
     const double fc = 0.5 * (lo + hi) * dt_ps / kPlanck_meV_ps;
+    const FormCost cost(p, s);
+    const int most = std::min(s.ring, s.T);
     for (int B : {32, 64, 128}) {
         if (only && B != only) continue;
         if (!project_shape_ok(B, 8, split) || (s.needs_acc && s.ring % B)) continue;   // flushes end between blocks
+        // no basis, tables or memory for what no push would use (its contraction taken to cost nothing, then what
+        // it costs): on small plans the launches' difference alone decides, and these are most of their creation
+        if (!only && !ever_picked(cost, B, 0.0, most)) continue;
         int R = 0;
         const std::vector<double> &basis = cache.basis(B, std::max(beta, 1e-6), 8, 48, &R);
         if (basis.empty() || !project_shape_ok(B, R, split)) continue;
@@ -297,6 +335,7 @@ tacaw_status build_band_forms(tacaw_plan_s *p, Stream &s, int64_t room_bytes, Ba
         b.work = (double)R / B * s.Nw_pad;
         std::vector<double> centre, w;
         if (split) w = choose_levels(s, b, &centre, cache);
+        if (!only && !ever_picked(cost, B, b.work, most)) continue;
         // one allocation: twiddles, first-level table, responses (FP64), basis (FP64), modulation, the second
         // level's basis, group centres and each energy's
         const int K = b.S ? b.r : R;
@@ -363,26 +402,20 @@ tacaw_status build_band_forms(tacaw_plan_s *p, Stream &s, int64_t room_bytes, Ba
     return TACAW_OK;
 }
 
-// The form with the least time a (row, frame), in picoseconds, fitted to measurements (2^16 to 2^20 rows, 8 to
-// 64 frames a push, 60 to 1000 energies): a push of frames 2.65 + 8 / n and 3 us a launch (0.5 more where it
-// parts the 16-byte chunks of 4 frames); a push of whole blocks 2.3 + 8 / n and 4 us a launch, and 3.7 for
-// the share of the frames that passes through the carry; the contraction 0.0139 (split) or 0.142 (FP32) a
-// product, a tenth more on coefficients (shorter sums, drained more often).  Both sides at the line: six
-// partitions pushed 16 frames at a time, 300 energies: frames 14.9 + 20.1 ms, blocks of 32 with
-// half their frames carried 21.2 + 11.0 ms.
+void share_band_forms(const Stream &from, Stream &s) {
+    std::copy(from.band, from.band + kBandForms, s.band);
+    s.n_band = from.n_band;
+    s.shift_mean = from.shift_mean;
+}
+
+// The form with the least time (FormCost).  Both sides at the line: six partitions pushed 16 frames at a time,
+// 300 energies: frames 14.9 + 20.1 ms, blocks of 32 with half their frames carried 21.2 + 11.0 ms.
 int choose_form(const tacaw_plan_s *p, const Stream &s, int n, bool band_only) {
-    const bool split = p->prec == TACAW_PREC_SPLIT_BF16;
-    const double product = split ? 0.0139 : 0.142, push_rows = (double)s.M * n;
-    double best = 0.97 * (2.65 + 8.0 / n + 3e6 / push_rows + (n % 4 ? 0.5 : 0.0) + product * s.Nw_pad);
-    if (band_only) best = HUGE_VAL;
+    const FormCost c(p, s);
+    double best = band_only ? HUGE_VAL : c.frames(n);
     int form = -1;
     for (int i = 0; i < s.n_band; ++i) {
-        const BandForm &b = s.band[i];
-        // share of the frames that wait in the carry, taking the ring's other pushes to be like its first:
-        // none for whole blocks, all but the completing push's for parts of a block, all for other sizes
-        // below a block (they drift against the blocks), a block's worth for longer ones
-        const double f = n % b.B == 0 ? 0.0 : b.B % n == 0 ? 1.0 - (double)n / b.B : n < b.B ? 1.0 : (double)b.B / n;
-        const double cost = 2.3 + 8.0 / std::max(n, 32) + 4e6 / push_rows + 3.7 * f + 1.1 * product * b.work;
+        const double cost = c.blocks(n, s.band[i].B, s.band[i].work);
         if (cost < best) {
             best = cost;
             form = i;

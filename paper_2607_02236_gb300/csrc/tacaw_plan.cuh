@@ -242,6 +242,8 @@ struct BandCache {
 // device memory; a stream without any keeps staging frames.  only: just the form with blocks of that many frames.
 tacaw_status build_band_forms(tacaw_plan_s *p, Stream &s, int64_t room_bytes, BandCache &cache, cudaStream_t st,
                               int only = 0);
+// Gives stream s the forms of `from`, a lane of the same Welch average.
+void share_band_forms(const Stream &from, Stream &s);
 // The staging form a ring takes whose first push has n frames (-1: frames, unless band_only and s has a form).
 int choose_form(const tacaw_plan_s *p, const Stream &s, int n, bool band_only = false);
 // Table arguments of stream s after its tables were built.

@@ -332,18 +332,19 @@ tacaw_status tacaw_restore_state(tacaw_plan_t p, const void *h_state, int64_t by
     // a ring in a form whose tables this plan had no room for at its creation: they are built now
     BandCache bases;
     for (size_t i = 0; i < p->s.size(); ++i) {
-        // (a split-FP16 segment without its kept mean goes on in coefficients)
-        if (p->f16 && (cnt[i].due & 2) && cnt[i].form == 0 && p->s[i].n_band == 0) {
-            c = build_band_forms(p, p->s[i], INT64_MAX, bases, st);
+        Stream &first = p->s[i - p->s[i].lane];   // the lanes of a Welch average share their tables
+        const int B = cnt[i].form;
+        // (a split-FP16 segment without its kept mean goes on in coefficients, of any form)
+        const bool any = B == 0 && p->f16 && (cnt[i].due & 2) && first.n_band == 0;
+        if (!any && (B == 0 || band_of(first, B) >= 0)) continue;
+        for (int b : {32, 64, 128}) {
+            if (any ? first.n_band > 0 : b != B) continue;
+            c = build_band_forms(p, first, INT64_MAX, bases, st, b);
             if (c != TACAW_OK) return c;
-            if (p->s[i].n_band == 0) return fail(TACAW_ERR_OOM, "checkpoint: no memory for stream %zu's band-limited forms", i);
         }
-        if (cnt[i].form == 0 || band_of(p->s[i], cnt[i].form) >= 0) continue;
-        c = build_band_forms(p, p->s[i], INT64_MAX, bases, st, cnt[i].form);
-        if (c != TACAW_OK) return c;
-        if (band_of(p->s[i], cnt[i].form) < 0)
-            return fail(TACAW_ERR_OOM, "checkpoint: no memory for the tables of stream %zu's blocks of %d frames", i,
-                        cnt[i].form);
+        if (any ? first.n_band == 0 : band_of(first, B) < 0)
+            return fail(TACAW_ERR_OOM, "checkpoint: no memory for the tables of stream %zu's blocks of frames", i);
+        for (int l = 1; l < p->us[first.user].lanes; ++l) share_band_forms(first, (&first)[l]);
     }
     if (state_total(p, cnt) != h.total_bytes)
         return fail(TACAW_ERR_INVALID_ARG, "checkpoint: section sizes do not match its counters");

@@ -346,3 +346,46 @@ def test_split_fp16_kept_mean_range(first, ring):
             fr[t] = bad
             plan.close()
             plan.__init__([cfg], precision="split_fp16", k_stage=512)
+
+
+def device_bytes(cfg, **kw):
+    from paper_2607_02236_gb300 import TacawPlan
+    with TacawPlan([cfg], **kw) as plan:
+        return plan.info()["device_bytes"]
+
+
+def test_tables_only_for_forms_a_push_can_take_and_once_a_stream():
+    """Few rows: no push length makes a form worth its launches, so none is built.  The lanes of a Welch average
+    share one set of tables."""
+    kw = dict(precision="split_bf16")
+    small = config(1024, 60, 120.0, kx=36, ky=13, pitch_row=36, pitch_frame=468, pitch_probe=468)
+    assert device_bytes(small, k_stage=1024, **kw) == device_bytes(small, **no_room(small, 1024, **kw))
+    tables = []
+    for stride in (256, 128):               # 2 and 4 lanes
+        cfg = config(512, 1000, 150.0, welch_segments=5, welch_stride=stride)
+        tables.append(device_bytes(cfg, k_stage=512, **kw) - device_bytes(cfg, **no_room(cfg, 512, **kw)))
+    assert tables[0] == tables[1] > 0
+
+
+@pytest.mark.parametrize("precision", ["split_bf16", "split_fp16", "fp32"])
+@pytest.mark.parametrize("mean", [True, False])
+def test_welch_lanes_in_blocks(precision, mean):
+    """Overlapping Welch segments that take the form, pushes of whole blocks of every lane."""
+    import torch
+    from paper_2607_02236_gb300 import TacawPlan
+    cfg = config(512, 1000, 150.0, welch_segments=3, welch_stride=256, subtract_mean=mean)
+    n = 2 * 256 + 512
+    fr = waves(n, 23)
+    with TacawPlan([cfg], precision=precision) as plan:
+        push_all(plan, fr, [64], 0, 320)
+        B = 128 if precision == "fp32" else 64
+        assert [ring_form(plan, i) for i in range(2)] == [B, B]
+        state = plan.save_state()
+        push_all(plan, fr, [64], 320)
+        I, _ = finish(plan)
+    with TacawPlan([cfg], **no_room(cfg, 512, precision=precision)) as plan:
+        plan.restore_state(state)           # builds the lanes' tables
+        push_all(plan, fr, [64], 320)
+        assert rel_err_peak(finish(plan)[0], I) <= TOL
+    ref = oracle.welch_forward(fr[:, PIX].cpu().numpy()[None, :, None, :], 512, 256, E_meV=cfg.E_meV, subtract_mean=mean)
+    assert rel_err_peak(I[:, PIX], ref.I[0, :, 0]) <= TOL
