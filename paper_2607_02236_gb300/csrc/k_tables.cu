@@ -259,16 +259,25 @@ __global__ void band_growth_kernel(int B, int per, int n, int total, const float
     }
 }
 
+// (c, s) of the next place along an even grid of angles: rotation by the step's (cd, sd), whose FP64 rounding over up
+// to 512 steps stays below 1e-13 (an FP64 sincospi at each was most of the tables' time)
+__device__ __forceinline__ void rotate(double &c, double &s, double cd, double sd) {
+    const double x = c * cd - s * sd;
+    s = s * cd + c * sd;
+    c = x;
+}
+
 // one thread per (energy, basis vector); a.cj holds c_j for FFT grids too
 __global__ void band_response_kernel(TableArgs a, BandTableArgs b, double *q_resp) {
     const int j = blockIdx.x * blockDim.x + threadIdx.x, q = blockIdx.y;
     if (j >= a.Nw) return;
     const double d = a.cj[j] - (b.fcj ? b.fcj[j] : b.fc);
-    double acc = 0.0;
+    double acc = 0.0, c, s, cd, sd;
+    sincospi(-d * (double)(b.B - 1), &s, &c);
+    sincospi(2.0 * d, &sd, &cd);
     for (int u = 0; u < b.B / 2; ++u) {
-        double c, s;
-        sincospi(2.0 * d * ((double)u - 0.5 * (double)(b.B - 1)), &s, &c);
         acc += b.basis[u * b.R + q] * (q >= b.R / 2 ? -2.0 * s : 2.0 * c);
+        rotate(c, s, cd, sd);
     }
     q_resp[(size_t)q * a.Nw + j] = acc;
 }
@@ -336,17 +345,17 @@ __global__ void band_merge_kernel(BandMergeArgs m, __nv_bfloat16 *T_hi, __nv_bfl
         const int g = col / m.r, p = col % m.r, k = slot / R, q = slot % R;
         const double fg = m.fg[g], c0 = 0.5 * (double)(B - 1);
         const bool odd_v = q >= R / 2, odd_w = p >= m.r / 2;
-        double sr = 0.0, si = 0.0;
+        double sr = 0.0, si = 0.0, s, c, sd, cd;
+        sincospi(-2.0 * (m.b.fc - fg) * c0, &s, &c);
+        sincospi(2.0 * (m.b.fc - fg), &sd, &cd);
         for (int u = 0; u < B; ++u) {
             const double v = u < B / 2 ? m.b.basis[u * R + q] : (odd_v ? -1.0 : 1.0) * m.b.basis[(B - 1 - u) * R + q];
             const int t = k * B + u;
             const double w = t < m.S / 2 ? m.w[t * m.r + p] : (odd_w ? -1.0 : 1.0) * m.w[(m.S - 1 - t) * m.r + p];
-            double s, c;
-            sincospi(2.0 * (m.b.fc - fg) * ((double)u - c0), &s, &c);
             sr += v * w * c;
             si += v * w * s;
+            rotate(c, s, cd, sd);
         }
-        double s, c;
         sincospi(-2.0 * fg * ((double)(k * B) + c0 - 0.5 * (double)(m.S - 1)), &s, &c);
         ar = sr * c - si * s;
         ai = sr * s + si * c;

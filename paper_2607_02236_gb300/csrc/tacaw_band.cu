@@ -38,33 +38,39 @@ public:
     // first halves of the n most concentrated sequences, the whole sequences of unit norm (norm sqrt(1/2))
     std::vector<std::vector<double>> vectors(int n) const {
         n = std::min(n, H);
-        // all eigenvalues side by side: each count is a chain of divisions, which the others overlap
-        std::vector<double> a(n, lo), b(n, hi), q(n), x(n);
-        std::vector<int> above(n);
-        for (int i = 0; i < 32; ++i) {   // to 2^-32 of the range, far below the gaps (about range / B^2)
-            for (int k = 0; k < n; ++k) {
-                x[k] = 0.5 * (a[k] + b[k]);
-                q[k] = 1.0;
-                above[k] = 0;
-            }
-            for (int u = 0; u < H; ++u) {
-                const double o2 = o[u] * o[u];   // (o[0] = 0)
-                for (int k = 0; k < n; ++k) {
-                    double t = d[u] - x[k] - o2 / q[k];
-                    t = t == 0.0 ? 1e-300 : t;
-                    above[k] += t > 0.0;         // positive pivots of A - x: eigenvalues above x
-                    q[k] = t;
+        // all eigenvalues side by side, four to a pass: each count is a chain of divisions, which the others overlap
+        constexpr int L = 4;
+        const int m = (n + L - 1) / L * L;
+        std::vector<double> a(m, lo), b(m, hi);
+        for (int i = 0; i < 24; ++i) {   // to 2^-24 of the range, below the gaps (range / B and less) by 2^10 and more
+            for (int k0 = 0; k0 < m; k0 += L) {
+                double x[L], q[L], above[L];
+                for (int k = 0; k < L; ++k) {
+                    x[k] = 0.5 * (a[k0 + k] + b[k0 + k]);
+                    q[k] = 1.0;
+                    above[k] = 0.0;
                 }
+                for (int u = 0; u < H; ++u) {
+                    const double o2 = o[u] * o[u], du = d[u];   // (o[0] = 0)
+                    for (int k = 0; k < L; ++k) {
+                        double t = du - x[k] - o2 / q[k];
+                        t = t == 0.0 ? 1e-300 : t;
+                        above[k] += t > 0.0 ? 1.0 : 0.0;        // positive pivots of A - x: eigenvalues above x
+                        q[k] = t;
+                    }
+                }
+                for (int k = 0; k < L; ++k) (above[k] > k0 + k ? a : b)[k0 + k] = x[k];
             }
-            for (int k = 0; k < n; ++k) (above[k] > k ? a[k] : b[k]) = x[k];
         }
         std::vector<std::vector<double>> out;
+        Factors f;
         for (int k = 0; k < n; ++k) {
             const double shift = 0.5 * (a[k] + b[k]) + 1e-11 * (hi - lo);   // off the eigenvalue: the solves stay finite
             std::vector<double> v(H);
             for (int u = 0; u < H; ++u) v[u] = 1.0 + 0.01 * (u % 7);   // no symmetry that could hide a vector
-            for (int it = 0; it < 4; ++it) {
-                solve(shift, v);
+            f.factor(*this, shift);
+            for (int it = 0; it < 5; ++it) {
+                f.solve(v);
                 double s = 0.0;
                 for (double t : v) s += t * t;
                 for (double &t : v) t *= std::sqrt(0.5 / s);
@@ -78,42 +84,54 @@ private:
     int H;
     std::vector<double> d, o;
     double lo, hi;
-    // v <- (A - x)^-1 v, Gaussian elimination with row exchanges (three diagonals above)
-    void solve(double x, std::vector<double> &v) const {
-        std::vector<double> a(H), b(H, 0.0), c(H, 0.0);   // the current upper rows: a b c at columns u, u+1, u+2
-        double p = d[0] - x, q = H > 1 ? o[1] : 0.0;       // row u as eliminated so far
-        for (int u = 0; u < H; ++u) {
-            if (u + 1 == H) {
-                a[u] = p == 0.0 ? 1e-300 : p;
-                break;
+    // A - x by Gaussian elimination with row exchanges: the multiplier of each step, and the upper rows
+    // (1 / a, b, c at columns u, u+1, u+2)
+    struct Factors {
+        std::vector<double> m, r, b, c;
+        std::vector<char> swapped;
+        void factor(const Prolate &A, double x) {
+            const int H = A.H;
+            m.assign(H, 0.0);
+            r.assign(H, 0.0);
+            b.assign(H, 0.0);
+            c.assign(H, 0.0);
+            swapped.assign(H, 0);
+            double p = A.d[0] - x, q = H > 1 ? A.o[1] : 0.0;   // row u as eliminated so far
+            for (int u = 0; u + 1 < H; ++u) {
+                const double l = A.o[u + 1], dn = A.d[u + 1] - x, on = u + 2 < H ? A.o[u + 2] : 0.0;
+                if (std::fabs(p) >= std::fabs(l)) {
+                    r[u] = 1.0 / (p == 0.0 ? 1e-300 : p);
+                    b[u] = q;
+                    m[u] = l * r[u];
+                    p = dn - m[u] * q;
+                    q = on;
+                } else {
+                    swapped[u] = 1;
+                    r[u] = 1.0 / l;
+                    b[u] = dn;
+                    c[u] = on;
+                    m[u] = p * r[u];
+                    p = q - m[u] * dn;
+                    q = -m[u] * on;
+                }
             }
-            const double l = o[u + 1], dn = d[u + 1] - x, on = u + 2 < H ? o[u + 2] : 0.0;
-            if (std::fabs(p) >= std::fabs(l)) {
-                a[u] = p == 0.0 ? 1e-300 : p;
-                b[u] = q;
-                const double m = l / a[u];
-                p = dn - m * q;
-                q = on;
-                v[u + 1] -= m * v[u];
-            } else {
-                a[u] = l;
-                b[u] = dn;
-                c[u] = on;
-                const double m = p / l;
-                p = q - m * dn;
-                q = -m * on;
-                const double t = v[u];
-                v[u] = v[u + 1];
-                v[u + 1] = t - m * v[u];
+            r[H - 1] = 1.0 / (p == 0.0 ? 1e-300 : p);
+        }
+        // v <- (A - x)^-1 v
+        void solve(std::vector<double> &v) const {
+            const int H = (int)v.size();
+            for (int u = 0; u + 1 < H; ++u) {
+                if (swapped[u]) std::swap(v[u], v[u + 1]);
+                v[u + 1] -= m[u] * v[u];
+            }
+            for (int u = H - 1; u >= 0; --u) {
+                double t = v[u];
+                if (u + 1 < H) t -= b[u] * v[u + 1];
+                if (u + 2 < H) t -= c[u] * v[u + 2];
+                v[u] = t * r[u];
             }
         }
-        for (int u = H - 1; u >= 0; --u) {
-            double t = v[u];
-            if (u + 1 < H) t -= b[u] * v[u + 1];
-            if (u + 2 < H) t -= c[u] * v[u + 2];
-            v[u] = t / a[u];
-        }
-    }
+    };
 };
 
 // About the rank band_basis finds at kBandTol for x = beta B degrees of freedom (x from 1 to 50).
