@@ -236,12 +236,18 @@ struct FormCost {
     }
 };
 
-// Whether the rule can pick blocks of B over frames for a push of some length (a ring's first push has up to
-// `most` frames).  Beyond two blocks both the launches' difference and the share carried fall with n, so the
-// lengths up to there, the longest whole number of blocks and the four longest (chunks parted or not) decide.
-bool ever_picked(const FormCost &c, int B, double work, int most) {
-    auto picks = [&](int n) { return n > 0 && n <= most && c.blocks(n, B, work) < c.frames(n); };
-    for (int n = 1; n <= 2 * B; ++n)
+// Whether the rule can pick blocks of B over frames and over s's forms so far for a push of some length (a
+// ring's first push has up to `most` frames).  Beyond two blocks both the launches' difference and the shares
+// carried fall with n, so the lengths up to there, the longest whole number of blocks and the four longest
+// (chunks parted or not) decide.
+bool ever_picked(const FormCost &c, const Stream &s, int B, double work, int most) {
+    auto picks = [&](int n) {
+        if (n < 1 || n > most) return false;
+        double best = c.frames(n);
+        for (int i = 0; i < s.n_band; ++i) best = std::min(best, c.blocks(n, s.band[i].B, s.band[i].work));
+        return c.blocks(n, B, work) < best;
+    };
+    for (int n = 1; n <= 4 * B; ++n)
         if (picks(n)) return true;
     return picks(most / B * B) || picks(most) || picks(most - 1) || picks(most - 2) || picks(most - 3);
 }
@@ -325,12 +331,16 @@ tacaw_status build_band_forms(tacaw_plan_s *p, Stream &s, int64_t room_bytes, Ba
     const double fc = 0.5 * (lo + hi) * dt_ps / kPlanck_meV_ps;
     const FormCost cost(p, s);
     const int most = std::min(s.ring, s.T);
-    for (int B : {32, 64, 128}) {
+    for (int B : {128, 64, 32}) {
         if (only && B != only) continue;
         if (!project_shape_ok(B, 8, split) || (s.needs_acc && s.ring % B)) continue;   // flushes end between blocks
-        // no basis, tables or memory for what no push would use (its contraction taken to cost nothing, then what
-        // it costs): on small plans the launches' difference alone decides, and these are most of their creation
-        if (!only && !ever_picked(cost, B, 0.0, most)) continue;
+        // no basis, tables or memory for what no push would use, first by the least work it could have (the rank is
+        // no more than 2 below the guess; two levels of ranks of 8), then by what it has: on small plans the
+        // launches' difference alone decides, and these are most of their creation
+        const double ratio = (double)std::max(8, rank_guess(beta * B) - 4) / B;
+        double least = ratio * s.Nw_pad;
+        if (split) least = std::min(least, ratio * 8 * s.n_wt + 8.0 / 512 * s.Nw_pad);
+        if (!only && !ever_picked(cost, s, B, least, most)) continue;
         int R = 0;
         const std::vector<double> &basis = cache.basis(B, std::max(beta, 1e-6), 8, 48, &R);
         if (basis.empty() || !project_shape_ok(B, R, split)) continue;
@@ -353,7 +363,7 @@ tacaw_status build_band_forms(tacaw_plan_s *p, Stream &s, int64_t room_bytes, Ba
         b.work = (double)R / B * s.Nw_pad;
         std::vector<double> centre, w;
         if (split) w = choose_levels(s, b, &centre, cache);
-        if (!only && !ever_picked(cost, B, b.work, most)) continue;
+        if (!only && !ever_picked(cost, s, B, b.work, most)) continue;
         // one allocation: twiddles, first-level table, responses (FP64), basis (FP64), modulation, the second
         // level's basis, group centres and each energy's
         const int K = b.S ? b.r : R;
