@@ -1023,13 +1023,14 @@ tacaw_status push_counted(tacaw_plan_s *p, UserStream &u, int n, cudaStream_t st
     return TACAW_OK;
 }
 
-// A ring's first push, of n frames: its form, and with a segment's first ring whether the provisional mean
-// leaves the frames.
-void start_ring(tacaw_plan_s *p, Stream &s, int n) {
+// A ring begins with the last `first` frames of a push of n: its form, and with a segment's first ring whether the
+// provisional mean leaves the frames.
+void start_ring(tacaw_plan_s *p, Stream &s, int n, int first) {
+    n = std::min(n, s.ring);
     // split FP16 with a kept mean: plain frames hold the mean (their residuals could leave the fp16 range that the
     // frames themselves are held to), coefficients do not, so a segment keeps to the kind its first ring has
     const bool one_kind = p->f16 && s.shift_mean && s.pushed > 0;
-    s.form = one_kind && !s.shifted ? -1 : choose_form(p, s, n, one_kind);
+    s.form = one_kind && !s.shifted ? -1 : choose_form(p, s, n, first, one_kind);
     if (s.pushed == 0) s.shifted = s.shift_mean && (!p->f16 || s.form >= 0);
 }
 
@@ -1065,15 +1066,16 @@ ProjEntry proj_entry(const tacaw_plan_s *p, const Stream &s, const FrameGeom &g,
     return e;
 }
 
-// Pushes n frames (device pointer, the stream's layout) into internal stream s.
-tacaw_status push_internal(tacaw_plan_s *p, Stream &s, const float2 *frames, int n_frames, cudaStream_t st) {
+// Pushes n frames (device pointer, the stream's layout) into internal stream s; push_len: frames of the caller's push
+// that they are of.
+tacaw_status push_internal(tacaw_plan_s *p, Stream &s, const float2 *frames, int n_frames, int push_len, cudaStream_t st) {
     const FrameGeom g = push_geom(s, frames);
     if (s.due) {
         // this stream's ring is full: its deferred flush (with any others) goes first
         tacaw_status r = flush_due(p, st);
         if (r != TACAW_OK) return r;
     }
-    if (s.staged == 0) start_ring(p, s, std::min(n_frames, s.ring));
+    if (s.staged == 0) start_ring(p, s, push_len, std::min(n_frames, s.ring));
     if (s.pushed == 0 && s.removes_mean()) {
         CU_CHECK(p, launch_mean(g, n_frames, s.mu_hat, st), "provisional mean");
         p->launches++;
@@ -1095,7 +1097,7 @@ tacaw_status push_internal(tacaw_plan_s *p, Stream &s, const float2 *frames, int
     int done = 0;
     while (done < n_frames) {
         const int chunk = std::min(n_frames - done, s.ring - s.staged);
-        if (s.staged == 0) start_ring(p, s, chunk);
+        if (s.staged == 0) start_ring(p, s, push_len, chunk);
         FrameGeom gc = g;
         gc.base = g.base + (int64_t)done * g.pitch_frame;
         if (p->in_place) {
@@ -1546,6 +1548,7 @@ tacaw_status validate_push(tacaw_plan_s *p, int sid, const void *d_frames, int n
 // One validated push of a user stream.
 tacaw_status push_user(tacaw_plan_s *p, int sid, const float2 *base, int n_frames, cudaStream_t st) {
     UserStream &u = p->us[sid];
+    const int push_len = n_frames;
     // leading frames of the stream that precede its first segment are dropped unread
     if (u.pushed + n_frames <= u.skip) {
         u.pushed += n_frames;
@@ -1558,7 +1561,7 @@ tacaw_status push_user(tacaw_plan_s *p, int sid, const float2 *base, int n_frame
         u.pushed = u.skip;
     }
     if (u.N <= 1) {
-        tacaw_status r = push_internal(p, p->s[u.first], base, n_frames, st);
+        tacaw_status r = push_internal(p, p->s[u.first], base, n_frames, push_len, st);
         if (r == TACAW_OK) u.pushed += n_frames;
         return r;
     }
@@ -1572,7 +1575,7 @@ tacaw_status push_user(tacaw_plan_s *p, int sid, const float2 *base, int n_frame
             const int64_t s0 = s.seg * (int64_t)u.stride;
             const int64_t lo = std::max(a, s0 + s.pushed), hi = std::min(b, s0 + u.L);
             if (lo >= hi) break;
-            tacaw_status r = push_internal(p, s, base + (lo - a) * s.d.pitch_frame, (int)(hi - lo), st);
+            tacaw_status r = push_internal(p, s, base + (lo - a) * s.d.pitch_frame, (int)(hi - lo), push_len, st);
             if (r != TACAW_OK) return r;
             if (s.pushed < s.T) break;
             r = finish_segment(p, u, s, st);
@@ -1634,7 +1637,7 @@ tacaw_status tacaw_push_frames_group(tacaw_plan_t p, int n, const int *stream_id
         const bool in_ring = u.N <= 1 && !p->in_place && !p->pipe && u.pushed >= u.skip && !s.due &&
                              s.staged + n_frames[i] <= s.ring;
         // the form is the ring's: its first push picks it, later ones continue it
-        if (in_ring && s.staged == 0) start_ring(p, s, n_frames[i]);
+        if (in_ring && s.staged == 0) start_ring(p, s, n_frames[i], n_frames[i]);
         banded[i] = in_ring && s.form >= 0;
         if (banded[i]) continue;
         if (in_ring && split && convert_split_groupable(p->bf, s.staged, n_frames[i])) {

@@ -227,11 +227,14 @@ struct FormCost {
     double frames(int n) const {
         return 0.97 * (2.65 + 8.0 / n + 3e6 / (rows * n) + (n % 4 ? 0.5 : 0.0) + product * Nw_pad);
     }
-    double blocks(int n, int B, double work) const {
-        // share of the frames that wait in the carry, taking the ring's other pushes to be like its first:
-        // none for whole blocks, all but the completing push's for parts of a block, all for other sizes
-        // below a block (they drift against the blocks), a block's worth for longer ones
-        const double f = n % B == 0 ? 0.0 : B % n == 0 ? 1.0 - (double)n / B : n < B ? 1.0 : (double)B / n;
+    // first: frames of the ring's first push (the end of one that began in the ring before it, or n)
+    double blocks(int n, int B, double work, int first) const {
+        // share of the frames that wait in the carry, taking the ring's other pushes to have n frames too: the first
+        // push's odd frames in each for whole blocks, all but the completing push's for parts of a block, all for
+        // other sizes below a block (they drift against the blocks), a block's worth for longer ones
+        const double f = n % B == 0 ? (double)(first % B) / n
+                         : B % n == 0 && first == n ? 1.0 - (double)n / B
+                         : n < B ? 1.0 : (double)B / n;
         return 2.3 + 8.0 / std::max(n, 32) + 4e6 / (rows * n) + 3.7 * f + 1.1 * product * work;
     }
 };
@@ -244,8 +247,8 @@ bool ever_picked(const FormCost &c, const Stream &s, int B, double work, int mos
     auto picks = [&](int n) {
         if (n < 1 || n > most) return false;
         double best = c.frames(n);
-        for (int i = 0; i < s.n_band; ++i) best = std::min(best, c.blocks(n, s.band[i].B, s.band[i].work));
-        return c.blocks(n, B, work) < best;
+        for (int i = 0; i < s.n_band; ++i) best = std::min(best, c.blocks(n, s.band[i].B, s.band[i].work, n));
+        return c.blocks(n, B, work, n) < best;
     };
     for (int n = 1; n <= 4 * B; ++n)
         if (picks(n)) return true;
@@ -438,12 +441,12 @@ void share_band_forms(const Stream &from, Stream &s) {
 
 // The form with the least time (FormCost).  Both sides at the line: six partitions pushed 16 frames at a time,
 // 300 energies: frames 14.9 + 20.1 ms, blocks of 32 with half their frames carried 21.2 + 11.0 ms.
-int choose_form(const tacaw_plan_s *p, const Stream &s, int n, bool band_only) {
+int choose_form(const tacaw_plan_s *p, const Stream &s, int n, int first, bool band_only) {
     const FormCost c(p, s);
     double best = band_only ? HUGE_VAL : c.frames(n);
     int form = -1;
     for (int i = 0; i < s.n_band; ++i) {
-        const double cost = c.blocks(n, s.band[i].B, s.band[i].work);
+        const double cost = c.blocks(n, s.band[i].B, s.band[i].work, first);
         if (cost < best) {
             best = cost;
             form = i;

@@ -244,8 +244,9 @@ tacaw_status build_band_forms(tacaw_plan_s *p, Stream &s, int64_t room_bytes, Ba
                               int only = 0);
 // Gives stream s the forms of `from`, a lane of the same Welch average.
 void share_band_forms(const Stream &from, Stream &s);
-// The staging form a ring takes whose first push has n frames (-1: frames, unless band_only and s has a form).
-int choose_form(const tacaw_plan_s *p, const Stream &s, int n, bool band_only = false);
+// The staging form of a ring that begins with `first` frames of a push of n (-1: frames, unless band_only and s has a
+// form).
+int choose_form(const tacaw_plan_s *p, const Stream &s, int n, int first, bool band_only = false);
 // Table arguments of stream s after its tables were built.
 TableArgs stream_table_args(const Stream &s, int block_frames);
 

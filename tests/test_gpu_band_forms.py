@@ -389,3 +389,22 @@ def test_welch_lanes_in_blocks(precision, mean):
         assert rel_err_peak(finish(plan)[0], I) <= TOL
     ref = oracle.welch_forward(fr[:, PIX].cpu().numpy()[None, :, None, :], 512, 256, E_meV=cfg.E_meV, subtract_mean=mean)
     assert rel_err_peak(I[:, PIX], ref.I[0, :, 0]) <= TOL
+
+
+def test_a_push_across_a_ring_end_keeps_the_form():
+    """Pushes of 96 frames into rings of 512: the second ring begins with 64 frames of one.  Its form is that of pushes
+    of 96 (blocks of 32), not of 64 (blocks of 64), into which every later push would end."""
+    from paper_2607_02236_gb300 import TacawPlan
+    cfg = config(1024, 600, 150.0)
+    fr = waves(1024, 25)
+    with TacawPlan([cfg], precision="split_bf16", k_stage=512) as plan:
+        push_all(plan, fr, [96], 0, 96)
+        assert ring_form(plan) == 32
+        push_all(plan, fr, [96], 96, 576)
+        assert ring_form(plan) == 32
+        push_all(plan, fr, [96], 576)
+        I, _ = finish(plan)
+        assert_exact(I, fr, cfg)
+        plan.reset()
+        push_all(plan, fr, [64], 0, 64)
+        assert ring_form(plan) == 64
