@@ -80,7 +80,8 @@ PIX = np.r_[0:16, 1000:16000:997, ROWS - 16:ROWS]
 
 
 def assert_exact(I, fr, cfg, Psi=None):
-    kw = dict(window_kind=cfg.window, window_param=cfg.window_param, E_meV=cfg.E_meV, subtract_mean=cfg.subtract_mean)
+    kw = dict(window_kind=cfg.window, window_param=cfg.window_param, E_meV=cfg.E_meV, fft_bins=cfg.fft_bins,
+              subtract_mean=cfg.subtract_mean)
     psi, want = oracle.forward_pixels(fr[:, PIX].cpu().numpy(), **kw)
     e = rel_err_peak(I[:, PIX], want)
     assert e <= TOL, e
@@ -408,3 +409,150 @@ def test_a_push_across_a_ring_end_keeps_the_form():
         plan.reset()
         push_all(plan, fr, [64], 0, 64)
         assert ring_form(plan) == 64
+
+
+PRECISIONS = ["split_bf16", "split_fp16", "fp32"]
+
+# T, energies, E_max, push sizes, k_stage, accumulators, block length on the split and on the FP32 path
+CASES = [(1000, 1000, 150.0, [64], 0, "auto", 64, 128),             # a last block of 40 (104) frames
+         (1025, 1000, 150.0, [64], 0, "auto", 64, 128),             # ... of one frame
+         (1023, 1000, 150.0, [100, 28], 0, "auto", 64, 128),        # ... of all but one; pushes that end inside blocks
+         (1000, 1000, 150.0, [63, 65, 1], 0, "auto", 64, 128),      # chunks of four frames parted
+         (1000, 1000, 150.0, [16], 0, "auto", 64, 128),             # three of four pushes only carry
+         (2081, 400, 120.0, [32], 0, "auto", 32, 128),              # split: two levels, a last superblock of 33 frames
+         (2081, 1000, 150.0, [64], 0, "auto", 64, 128),             # split: two levels, superblocks of 512
+         (1000, 700, 60.0, [64], 0, "auto", 64, 128),               # small ranks, two levels
+         (1024, 1000, 240.0, [64], 0, "auto", 64, 64),              # the greatest rank of the split path
+         (2048, 1000, 150.0, [64], 512, "kahan", 64, 128),          # four flushes
+         (2048, 400, 120.0, [32], 512, "fp32", 32, 128),
+         (1152, 1000, 150.0, [96], 384, "fp64", 64, 128)]           # pushes across the rings' ends
+
+
+@pytest.mark.parametrize("precision", PRECISIONS)
+@pytest.mark.parametrize("case", range(len(CASES)))
+def test_forms_against_the_oracle(case, precision):
+    from paper_2607_02236_gb300 import TacawPlan
+    T, nw, E_max, sizes, k_stage, accum, split, fp32 = CASES[case]
+    cfg = config(T, nw, E_max, window=("hann", "gauss", "rect")[case % 3], window_param=T / 6.0 if case % 3 == 1 else 0.0,
+                 subtract_mean=case % 4 != 1)
+    fr = waves(T, 30 + case)
+    with TacawPlan([cfg], precision=precision, k_stage=k_stage, accum=accum) as plan:
+        push_all(plan, fr, sizes, 0, sizes[0])
+        assert ring_form(plan) == (fp32 if precision == "fp32" else split)
+        push_all(plan, fr, sizes[1:] + sizes[:1], sizes[0])
+        I, Psi = finish(plan, psi=True)
+        if k_stage:
+            assert plan.info()["flushes"] == -(-T // k_stage)
+    assert_exact(I, fr, cfg, Psi)
+
+
+@pytest.mark.parametrize("precision", PRECISIONS)
+@pytest.mark.parametrize("grid", ["signed", "uneven", "offset", "fft"])
+def test_energy_grids_in_blocks(grid, precision):
+    from paper_2607_02236_gb300 import TacawPlan
+    T = 4000 if grid == "fft" else 768
+    rng = np.random.default_rng(3)
+    E = {"signed": np.linspace(-90.0, 90.0, 600), "uneven": rng.permutation(120.0 * (np.arange(600) / 600.0) ** 2),
+         "offset": np.linspace(40.0, 160.0, 600), "fft": None}[grid]
+    cfg = config(T, 600, 120.0, subtract_mean=grid != "offset")
+    cfg.E_meV, cfg.fft_bins = (None, 900) if E is None else ([float(e) for e in E], 0)
+    fr = waves(T, 40)
+    with TacawPlan([cfg], precision=precision) as plan:
+        push_all(plan, fr, [64], 0, 64)
+        assert ring_form(plan) == (128 if precision == "fp32" else 64)
+        push_all(plan, fr, [64], 64)
+        I, Psi = finish(plan, psi=True)
+    assert_exact(I, fr, cfg, Psi)
+
+
+@pytest.mark.parametrize("precision", PRECISIONS)
+def test_groups_and_checkpoints_of_streams_in_blocks(precision):
+    """Two streams of different length, pushes that end inside blocks, two rings a segment: group pushes and a
+    checkpoint with unfinished blocks give the bits of single pushes, and the checkpoint is smaller than the frames
+    it stands for."""
+    import torch
+    from paper_2607_02236_gb300 import TacawPlan
+    cfgs = [config(1024, 1000, 150.0), config(768, 1000, 150.0, subtract_mean=False)]    # rings of 512 and 384
+    frs = [waves(1024, 51), waves(768, 52)]
+    sizes = [48, 80]
+
+    def rounds(plan, a, b, grouped):
+        done = [0, 0]
+        for r in range(b):
+            todo = [(i, done[i], min(sizes[r % 2], c.T - done[i])) for i, c in enumerate(cfgs) if done[i] < c.T]
+            for i, _, n in todo:
+                done[i] += n
+            if r < a:
+                continue
+            if grouped:
+                plan.push_group([i for i, _, _ in todo], [at(frs[i], t) for i, t, _ in todo], [n for _, _, n in todo])
+            else:
+                for i, t, n in todo:
+                    plan.push(i, at(frs[i], t), n)
+        return done
+
+    def outputs(plan):
+        I = torch.zeros(plan.info()["I_elems"], device="cuda")
+        plan.finalize(I)
+        return I.cpu().numpy().reshape(2, -1, ROWS)
+
+    kw = dict(precision=precision, k_stage=512, accum="kahan")
+    with TacawPlan(cfgs, **kw) as plan:
+        rounds(plan, 0, 16, False)
+        ref = outputs(plan)
+        plan.reset()
+        rounds(plan, 0, 16, True)
+        assert np.array_equal(outputs(plan), ref)
+        for cut_at in (3, 5, 9):            # 176, 304 (in the first rings) and 560 frames
+            plan.reset()
+            done = rounds(plan, 0, cut_at, True)
+            state = plan.save_state()
+            B = 128 if precision == "fp32" else 64
+            assert [ring_form(plan, i) for i in range(2)] == [B, B]
+            pad = -(-ROWS // 128) * 128
+            if cut_at < 9:
+                assert state.size < sum(24 * ROWS + 8 * d * pad for d in done)
+            with TacawPlan(cfgs, **kw) as other:
+                other.restore_state(state)
+                rounds(other, cut_at, 16, False)
+                assert np.array_equal(outputs(other), ref)
+    for i, (cfg, fr) in enumerate(zip(cfgs, frs)):
+        assert_exact(ref[i], fr, cfg)
+
+
+@pytest.mark.parametrize("precision", PRECISIONS)
+def test_captured_segment_in_blocks(precision):
+    """A segment in blocks captured into a graph: replays on new frames give the bits of eager passes."""
+    import torch
+    from paper_2607_02236_gb300 import TacawPlan
+    cfg = config(2081, 400, 120.0, subtract_mean=False)
+    frs = [waves(2081, 61), waves(2081, 62)]
+    buf = frs[0].clone()
+    st = torch.cuda.Stream()
+    with TacawPlan([cfg], precision=precision) as plan:
+        I = torch.zeros(plan.info()["I_elems"], device="cuda")
+
+        def segment():
+            plan.reset(st)
+            for t in range(0, 2081, 32):
+                plan.push(0, at(buf, t), min(32, 2081 - t), st)
+            plan.finalize_async(I, None, None, st)
+
+        want = []
+        for fr in frs:
+            buf.copy_(fr)
+            torch.cuda.synchronize()
+            segment()
+            plan.check_errors(st)
+            want.append(I.cpu().numpy().copy())
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=st):
+            segment()
+        for k in (1, 0, 1):
+            buf.copy_(frs[k])
+            I.zero_()
+            torch.cuda.synchronize()
+            graph.replay()
+            torch.cuda.synchronize()
+            assert np.array_equal(I.cpu().numpy(), want[k])
+    assert_exact(want[1].reshape(-1, ROWS), frs[1], cfg)
