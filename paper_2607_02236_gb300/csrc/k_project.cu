@@ -56,10 +56,12 @@ __device__ __forceinline__ void proj_copy(float2 *dst, const float2 *src, int by
 }
 
 // tot + rest += part, the rounding of tot kept in rest (Knuth's two-sum).  The residual sums behind the exact
-// mean run in FP32 over a few frames only, as in the conversions of plain frames (up to 32 on the split path, 8
-// on the FP32 path), and are exact from there on.  On the FP32 path a block has up to 16 such partial sums: FP64
-// adds would be two additions and two conversions each, on a pipe with a 64th of the FP32 rate; this costs the
-// FP32 scan (blocks of 128 frames, R 36) 6.10 ms instead of 6.05.
+// mean round no more than those of plain frames, which go to FP64 after 8 frames (FP32 path) or 32 (split path).
+// On the FP32 path a block has up to 16 sums of eight frames: FP64 adds would be two additions and two conversions
+// each, on a pipe with a 64th of the FP32 rate; this costs the FP32 scan (blocks of 128 frames, R 36) 6.10 ms instead
+// of 6.05.  On the split path a block's 8 or 16 sums of four frames are added in FP32: with frames of size a and
+// unit rounding u, at most (16 9 + 4 (1 + .. + 16)) a u = 688 a u for 64 frames, where two sums of 32 frames one by
+// one have 1054 a u.
 __device__ __forceinline__ void add_partial(float2 &tot, float2 &rest, float2 part) {
     const float2 t = __fadd2_rn(tot, part);
     const float2 b = __fadd2_rn(t, make_float2(-tot.x, -tot.y));       // the part as it went in
@@ -148,10 +150,10 @@ struct ProjSmem {
 // 2048 frames, bf16 pieces of the frames 0.5e-6); the fp16 range is met by a power-of-two scale per
 // row, taken from the ring's first nonzero block and the window (row_scale_for) and undone in the
 // contraction's epilogue.  A row that outgrows it has its staged coefficients rescaled.
-// CHECK: frame components beyond 65504 / e.f16_scale set DEVERR_FP16_RANGE (split-FP16 plans): of the frames less
-// their provisional mean, as those of plain frames, or with e.check_raw as they are (a kept mean stays in plain frames).
+// CHECK: frame components beyond 65504 / e.f16_scale set DEVERR_FP16_RANGE (split-FP16 plans): 1: of the frames less
+// their provisional mean, as those of plain frames; 2: of the frames as they are (a kept mean stays in plain frames).
 // ONE: a launch of one entry, whose fields then are constants of the launch and not loads by index.
-template <int B, int R, bool SPLIT, bool CHECK, bool ONE>
+template <int B, int R, bool SPLIT, int CHECK, bool ONE>
 __global__ void __launch_bounds__(128, ProjSmem<B, R, SPLIT>::kCtas)
     project_group_kernel(const __grid_constant__ ProjGroup pg) {
     using SM = ProjSmem<B, R, SPLIT>;
@@ -268,8 +270,7 @@ __global__ void __launch_bounds__(128, ProjSmem<B, R, SPLIT>::kCtas)
             const bool whole = f0 >= 0 && f0 + B <= e.n;
             // coefficient pairs (2 i, 2 i + 1) of the even and the odd half
             float2 er[RP], ei[RP], dr[RP], di[RP];
-            // sums of the residuals: SPLIT: tot of the block's first half, sum of its second; else add_partial's
-            float2 sum = make_float2(0.f, 0.f), tot = sum, rest = sum;
+            float2 tot = make_float2(0.f, 0.f), rest = tot;   // sum of the residuals (rest: add_partial's)
 #pragma unroll
             for (int i = 0; i < RP; ++i) er[i] = ei[i] = dr[i] = di[i] = make_float2(0.f, 0.f);
 #pragma unroll 1
@@ -281,18 +282,19 @@ __global__ void __launch_bounds__(128, ProjSmem<B, R, SPLIT>::kCtas)
                 get = (get + 1) % NS;
                 copy_stage();                     // into the slot read one stage ago
                 const float2 nmu = make_float2(-mu.x, -mu.y);
-                if (CHECK && e.check_raw) {       // (carried frames were checked when they came)
+                if (CHECK == 2) {                 // (carried frames were checked when they came)
 #pragma unroll
                     for (int i = 0; i < 2 * KP; ++i) {
                         const int f = f0 + (i < KP ? KP * st + i : B - 1 - KP * st - (i - KP));
                         if (f >= 0) amax = fmaxf(amax, fmaxf(fabsf(y[i].x), fabsf(y[i].y)));
                     }
                 }
+                float2 part = make_float2(0.f, 0.f);
                 if (whole) {
 #pragma unroll
                     for (int i = 0; i < 2 * KP; ++i) {
                         y[i] = __fadd2_rn(y[i], nmu);
-                        (SPLIT && i < KP ? tot : sum) = __fadd2_rn(SPLIT && i < KP ? tot : sum, y[i]);
+                        part = __fadd2_rn(part, y[i]);
                     }
                 } else {
 #pragma unroll
@@ -300,15 +302,13 @@ __global__ void __launch_bounds__(128, ProjSmem<B, R, SPLIT>::kCtas)
                         const int f = f0 + (i < KP ? KP * st + i : B - 1 - KP * st - (i - KP));
                         if (f >= 0 && f < e.n) {   // (carried frames are residuals, already counted)
                             y[i] = __fadd2_rn(y[i], nmu);
-                            (SPLIT && i < KP ? tot : sum) = __fadd2_rn(SPLIT && i < KP ? tot : sum, y[i]);
+                            part = __fadd2_rn(part, y[i]);
                         }
                     }
                 }
-                if (!SPLIT) {                     // (eight frames a stage)
-                    add_partial(tot, rest, sum);
-                    sum = make_float2(0.f, 0.f);
-                }
-                if (CHECK && !e.check_raw) {
+                if (SPLIT) tot = __fadd2_rn(tot, part);
+                else add_partial(tot, rest, part);
+                if (CHECK == 1) {
 #pragma unroll
                     for (int i = 0; i < 2 * KP; ++i) amax = fmaxf(amax, fmaxf(fabsf(y[i].x), fabsf(y[i].y)));
                 }
@@ -353,7 +353,7 @@ __global__ void __launch_bounds__(128, ProjSmem<B, R, SPLIT>::kCtas)
                     }
                 }
             }
-            if ((int64_t)m < e.g.M) add_residual(&e.sum_res[m], tot, SPLIT ? sum : rest);
+            if ((int64_t)m < e.g.M) add_residual(&e.sum_res[m], tot, rest);
             // coefficient q of the block: even half first
             auto z = [&](int q) {
                 const int i = (q % RH) >> 1;
@@ -434,7 +434,7 @@ __global__ void __launch_bounds__(128, ProjSmem<B, R, SPLIT>::kCtas)
                         const float2 y = make_float2(v[i].x - mu.x, v[i].y - mu.y);
                         sum = __fadd2_rn(sum, y);
                         if (CHECK) {
-                            const float2 c = e.check_raw ? v[i] : y;
+                            const float2 c = CHECK == 2 ? v[i] : y;
                             amax = fmaxf(amax, fmaxf(fabsf(c.x), fabsf(c.y)));
                         }
                         carry[(int64_t)(base + f + i) * e.M_pad] = y;
@@ -449,7 +449,7 @@ __global__ void __launch_bounds__(128, ProjSmem<B, R, SPLIT>::kCtas)
 
 // Pushes that complete no block: their frames' residuals go to the carry, 8 bytes read and 8 written a
 // (row, frame) at full occupancy.  CTA b: rows 128 (b - group_begin) .. of its entry.
-template <bool CHECK>
+template <int CHECK>
 __global__ void __launch_bounds__(128) carry_group_kernel(const __grid_constant__ ProjGroup pg) {
     int i = 0;
     while (i + 1 < pg.n && (int64_t)blockIdx.x >= pg.e[i + 1].group_begin) ++i;
@@ -473,7 +473,7 @@ __global__ void __launch_bounds__(128) carry_group_kernel(const __grid_constant_
                 const float2 y = make_float2(v[f].x - mu.x, v[f].y - mu.y);
                 sum[f / 8] = __fadd2_rn(sum[f / 8], y);
                 if (CHECK) {
-                    const float2 c = e.check_raw ? v[f] : y;
+                    const float2 c = CHECK == 2 ? v[f] : y;
                     amax = fmaxf(amax, fmaxf(fabsf(c.x), fabsf(c.y)));
                 }
                 carry[(int64_t)(f0 + f) * e.M_pad] = y;
@@ -485,10 +485,12 @@ __global__ void __launch_bounds__(128) carry_group_kernel(const __grid_constant_
     if (CHECK && amax * e.f16_scale > 65504.f) atomicOr(e.err, DEVERR_FP16_RANGE);
 }
 
-template <int B, int R, bool SPLIT, bool CHECK>
+template <int B, int R, bool SPLIT, int CHECK>
 static cudaError_t launch_project_kernel(const ProjGroup &pg, cudaStream_t st) {
     using SM = ProjSmem<B, R, SPLIT>;
-    auto *kern = pg.n == 1 ? project_group_kernel<B, R, SPLIT, CHECK, true> : project_group_kernel<B, R, SPLIT, CHECK, false>;
+    auto *kern = project_group_kernel<B, R, SPLIT, CHECK, false>;
+    if constexpr (CHECK != 2)   // (rare: one kernel for any number of entries)
+        if (pg.n == 1) kern = project_group_kernel<B, R, SPLIT, CHECK, true>;
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -504,10 +506,11 @@ static cudaError_t launch_project_kernel(const ProjGroup &pg, cudaStream_t st) {
 template <int B, int R>
 static cudaError_t launch_project_shape(const ProjGroup &pg, bool split, cudaStream_t st) {
     if constexpr (B == 32 || (B == 64 && R <= 36)) {
-        if (split && pg.e[0].err) return launch_project_kernel<B, R, true, true>(pg, st);
-        if (split) return launch_project_kernel<B, R, true, false>(pg, st);
+        if (split && pg.check == 2) return launch_project_kernel<B, R, true, 2>(pg, st);
+        if (split && pg.check == 1) return launch_project_kernel<B, R, true, 1>(pg, st);
+        if (split) return launch_project_kernel<B, R, true, 0>(pg, st);
     }
-    if constexpr (B >= 64) return launch_project_kernel<B, R, false, false>(pg, st);
+    if constexpr (B >= 64) return launch_project_kernel<B, R, false, 0>(pg, st);
     return cudaErrorInvalidValue;
 }
 
@@ -532,10 +535,12 @@ cudaError_t launch_project_group(ProjGroup &pg, int B, int R, bool split, cudaSt
     bool blocks = false;
     for (int i = 0; i < pg.n; ++i) blocks = blocks || pg.e[i].nblk > 0;
     if (!blocks) {
-        if (pg.e[0].err)
-            carry_group_kernel<true><<<(unsigned)pg.groups, 128, 0, st>>>(pg);
+        if (pg.check == 2)
+            carry_group_kernel<2><<<(unsigned)pg.groups, 128, 0, st>>>(pg);
+        else if (pg.check == 1)
+            carry_group_kernel<1><<<(unsigned)pg.groups, 128, 0, st>>>(pg);
         else
-            carry_group_kernel<false><<<(unsigned)pg.groups, 128, 0, st>>>(pg);
+            carry_group_kernel<0><<<(unsigned)pg.groups, 128, 0, st>>>(pg);
         return cudaGetLastError();
     }
 #define TACAW_PROJ(b, r) \

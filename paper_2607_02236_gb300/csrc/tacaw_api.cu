@@ -1034,6 +1034,9 @@ void start_ring(tacaw_plan_s *p, Stream &s, int n, int first) {
     if (s.pushed == 0) s.shifted = s.shift_mean && (!p->f16 || s.form >= 0);
 }
 
+// The range check of a stream's frames (ProjGroup::check).
+int range_check(const tacaw_plan_s *p, const Stream &s) { return !p->f16 ? 0 : s.d.subtract_mean ? 1 : 2; }
+
 // The conversion of one push of n frames (inside the ring) on the ring's band-limited form.
 ProjEntry proj_entry(const tacaw_plan_s *p, const Stream &s, const FrameGeom &g, int n) {
     const BandForm &b = s.band[s.form];
@@ -1058,11 +1061,8 @@ ProjEntry proj_entry(const tacaw_plan_s *p, const Stream &s, const FrameGeom &g,
     e.A32 = s.A32;
     e.row_scale = s.row_scale();
     e.growth = b.growth + (s.stage_start / b.B + blk0);
-    if (p->f16) {
-        e.f16_scale = p->f16_scale;
-        e.check_raw = !s.d.subtract_mean;
-        e.err = p->d_err;
-    }
+    e.f16_scale = p->f16_scale;
+    e.err = p->d_err;
     return e;
 }
 
@@ -1111,6 +1111,7 @@ tacaw_status push_internal(tacaw_plan_s *p, Stream &s, const float2 *frames, int
             if (s.form >= 0) {
                 ProjGroup pg;
                 pg.n = 1;
+                pg.check = range_check(p, s);
                 pg.e[0] = proj_entry(p, s, gc, chunk);
                 const BandForm &b = s.band[s.form];
                 std::copy(b.basis.begin(), b.basis.end(), pg.basis);
@@ -1653,12 +1654,15 @@ tacaw_status tacaw_push_frames_group(tacaw_plan_t p, int n, const int *stream_id
         const BandForm &b = p->s[p->us[stream_ids[i]].first].band[p->s[p->us[stream_ids[i]].first].form];
         ProjGroup pg;
         pg.n = 0;
+        pg.check = range_check(p, p->s[p->us[stream_ids[i]].first]);
         std::copy(b.basis.begin(), b.basis.end(), pg.basis);
         std::vector<int> ids;
         for (int k = i; k < n && pg.n < kConvGroupMax; ++k) {
             if (!banded[k]) continue;
             Stream &s = p->s[p->us[stream_ids[k]].first];
-            if (s.band[s.form].B != b.B || s.band[s.form].R != b.R || s.band[s.form].beta != b.beta) continue;
+            if (s.band[s.form].B != b.B || s.band[s.form].R != b.R || s.band[s.form].beta != b.beta ||
+                range_check(p, s) != pg.check)
+                continue;
             banded[k] = 0;
             ids.push_back(k);
             const FrameGeom g = push_geom(s, static_cast<const float2 *>(d_frames[k]));

@@ -351,18 +351,19 @@ struct ProjEntry {
     float *row_scale;          // split staging: [M_pad] scale of the row's staged coefficients (0: all zero so far)
     const unsigned char *growth;   // split staging: exponent of the window's growth from each completed block
                                    // to its largest in the ring
-    float f16_scale;           // split-FP16 plans: frames are checked against the fp16 range at this
-    uint32_t *err;             // scale (err not null), less their provisional mean, or with check_raw (a
-    int check_raw;             // stream that keeps its mean) as they are
+    float f16_scale;           // split-FP16 plans (ProjGroup::check): frames are checked against the fp16 range at
+    uint32_t *err;             // this scale
     int64_t group_begin;       // set by the launcher: first of its groups of 128 rows
 };
 struct ProjGroup {
     ProjEntry e[kConvGroupMax];
     int n;
+    int check;                 // range check: 0 none, 1 of the frames less their provisional mean, 2 of the
+                               // frames as they are (streams that keep their mean)
     int64_t groups;            // set by the launcher
     alignas(16) float basis[64 * 48];   // [B/2][R] rows of the block's first half: R/2 even vectors, R/2 odd
 };
-// one launch over the pushes of pg.n <= kConvGroupMax streams, all on the same basis: blocks of B
+// one launch over the pushes of pg.n <= kConvGroupMax streams, all on the same basis and with the same check: blocks of B
 // frames, R coefficients (a shape project_shape_ok accepts), pg.basis; split: fp16 hi/lo rows of 32 slots, else FP32
 cudaError_t launch_project_group(ProjGroup &pg, int B, int R, bool split, cudaStream_t st);
 bool project_shape_ok(int B, int R, bool split);
