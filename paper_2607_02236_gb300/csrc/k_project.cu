@@ -57,11 +57,10 @@ __device__ __forceinline__ void proj_copy(float2 *dst, const float2 *src, int by
 
 // tot + rest += part, the rounding of tot kept in rest (Knuth's two-sum).  The residual sums behind the exact
 // mean round no more than those of plain frames, which go to FP64 after 8 frames (FP32 path) or 32 (split path).
-// On the FP32 path a block has up to 16 sums of eight frames: FP64 adds would be two additions and two conversions
-// each, on a pipe with a 64th of the FP32 rate; this costs the FP32 scan (blocks of 128 frames, R 36) 6.10 ms instead
-// of 6.05.  On the split path a block's 8 or 16 sums of four frames are added in FP32: with frames of size a and
-// unit rounding u, at most (16 9 + 4 (1 + .. + 16)) a u = 688 a u for 64 frames, where two sums of 32 frames one by
-// one have 1054 a u.
+// With frames of size a and unit rounding u: on the FP32 path sums of 16 frames from four sums of four (68 a u, two sums
+// of eight one by one 70) are added this way; FP64 adds would be two additions and two conversions each, on a pipe with
+// a 64th of the FP32 rate.  On the split path a block's sums of four frames are added in FP32: 668 a u for 64 frames,
+// two sums of 32 one by one 1054.  Cost: the FP32 scan (blocks of 128 frames, R 36) 6.16 ms instead of 6.05.
 __device__ __forceinline__ void add_partial(float2 &tot, float2 &rest, float2 part) {
     const float2 t = __fadd2_rn(tot, part);
     const float2 b = __fadd2_rn(t, make_float2(-tot.x, -tot.y));       // the part as it went in
@@ -71,6 +70,10 @@ __device__ __forceinline__ void add_partial(float2 &tot, float2 &rest, float2 pa
     tot = t;
 }
 // (one lane alone adds to a row in a launch: the sum's order is fixed)
+__device__ __forceinline__ void add_residual(double2 *sum_res, float2 tot) {
+    atomicAdd(&sum_res->x, (double)tot.x);
+    atomicAdd(&sum_res->y, (double)tot.y);
+}
 __device__ __forceinline__ void add_residual(double2 *sum_res, float2 tot, float2 rest) {
     atomicAdd(&sum_res->x, (double)tot.x + (double)rest.x);
     atomicAdd(&sum_res->y, (double)tot.y + (double)rest.y);
@@ -270,7 +273,7 @@ __global__ void __launch_bounds__(128, ProjSmem<B, R, SPLIT>::kCtas)
             const bool whole = f0 >= 0 && f0 + B <= e.n;
             // coefficient pairs (2 i, 2 i + 1) of the even and the odd half
             float2 er[RP], ei[RP], dr[RP], di[RP];
-            float2 tot = make_float2(0.f, 0.f), rest = tot;   // sum of the residuals (rest: add_partial's)
+            float2 tot = make_float2(0.f, 0.f), rest = tot, part = tot;   // sum of the residuals (rest: add_partial's)
 #pragma unroll
             for (int i = 0; i < RP; ++i) er[i] = ei[i] = dr[i] = di[i] = make_float2(0.f, 0.f);
 #pragma unroll 1
@@ -289,12 +292,13 @@ __global__ void __launch_bounds__(128, ProjSmem<B, R, SPLIT>::kCtas)
                         if (f >= 0) amax = fmaxf(amax, fmaxf(fabsf(y[i].x), fabsf(y[i].y)));
                     }
                 }
-                float2 part = make_float2(0.f, 0.f);
+                float2 s0 = make_float2(0.f, 0.f), s1 = s0;   // residuals of the block's front and back frames
                 if (whole) {
 #pragma unroll
                     for (int i = 0; i < 2 * KP; ++i) {
                         y[i] = __fadd2_rn(y[i], nmu);
-                        part = __fadd2_rn(part, y[i]);
+                        float2 &s = i < KP ? s0 : s1;
+                        s = i % KP == 0 ? y[i] : __fadd2_rn(s, y[i]);
                     }
                 } else {
 #pragma unroll
@@ -302,12 +306,20 @@ __global__ void __launch_bounds__(128, ProjSmem<B, R, SPLIT>::kCtas)
                         const int f = f0 + (i < KP ? KP * st + i : B - 1 - KP * st - (i - KP));
                         if (f >= 0 && f < e.n) {   // (carried frames are residuals, already counted)
                             y[i] = __fadd2_rn(y[i], nmu);
-                            part = __fadd2_rn(part, y[i]);
+                            float2 &s = i < KP ? s0 : s1;
+                            s = __fadd2_rn(s, y[i]);
                         }
                     }
                 }
-                if (SPLIT) tot = __fadd2_rn(tot, part);
-                else add_partial(tot, rest, part);
+                if (SPLIT) {
+                    tot = __fadd2_rn(tot, __fadd2_rn(s0, s1));
+                } else {
+                    part = __fadd2_rn(part, __fadd2_rn(s0, s1));
+                    if (st & 1) {
+                        add_partial(tot, rest, part);
+                        part = make_float2(0.f, 0.f);
+                    }
+                }
                 if (CHECK == 1) {
 #pragma unroll
                     for (int i = 0; i < 2 * KP; ++i) amax = fmaxf(amax, fmaxf(fabsf(y[i].x), fabsf(y[i].y)));
@@ -353,7 +365,10 @@ __global__ void __launch_bounds__(128, ProjSmem<B, R, SPLIT>::kCtas)
                     }
                 }
             }
-            if ((int64_t)m < e.g.M) add_residual(&e.sum_res[m], tot, rest);
+            if ((int64_t)m < e.g.M) {
+                if (SPLIT) add_residual(&e.sum_res[m], tot);
+                else add_residual(&e.sum_res[m], tot, rest);
+            }
             // coefficient q of the block: even half first
             auto z = [&](int q) {
                 const int i = (q % RH) >> 1;
@@ -439,7 +454,7 @@ __global__ void __launch_bounds__(128, ProjSmem<B, R, SPLIT>::kCtas)
                         }
                         carry[(int64_t)(base + f + i) * e.M_pad] = y;
                     }
-                if (valid) add_residual(&e.sum_res[m], sum, make_float2(0.f, 0.f));
+                if (valid) add_residual(&e.sum_res[m], sum);
             }
         }
         if (CHECK && amax * e.f16_scale > 65504.f) atomicOr(e.err, DEVERR_FP16_RANGE);
@@ -448,9 +463,11 @@ __global__ void __launch_bounds__(128, ProjSmem<B, R, SPLIT>::kCtas)
 }
 
 // Pushes that complete no block: their frames' residuals go to the carry, 8 bytes read and 8 written a
-// (row, frame) at full occupancy.  CTA b: rows 128 (b - group_begin) .. of its entry.
-template <int CHECK>
-__global__ void __launch_bounds__(128) carry_group_kernel(const __grid_constant__ ProjGroup pg) {
+// (row, frame) at full occupancy; their sums to FP64 every 32 frames (SPLIT) or 8, straight to memory: kept in
+// registers over the push (add_partial) the longer code cost more than the atomics (16-frame pushes of 10^4 rows
+// x 2048 frames, FP32: 1.47 ms a segment against 1.30).  CTA b: rows 128 (b - group_begin) .. of its entry.
+template <int CHECK, bool SPLIT>
+__global__ void __launch_bounds__(128, 8) carry_group_kernel(const __grid_constant__ ProjGroup pg) {
     int i = 0;
     while (i + 1 < pg.n && (int64_t)blockIdx.x >= pg.e[i + 1].group_begin) ++i;
     const ProjEntry &e = pg.e[i];
@@ -460,37 +477,46 @@ __global__ void __launch_bounds__(128) carry_group_kernel(const __grid_constant_
     const float2 *src = e.g.base + proj_row(e.g, m);
     float2 *carry = e.carry + m + (int64_t)e.c0 * e.M_pad;
     const float2 mu = e.mu_hat[m];
-    float2 tot = make_float2(0.f, 0.f), rest = tot;
+    float2 sum = make_float2(0.f, 0.f), half = sum;
     float amax = 0.f;
     for (int f0 = 0; f0 < e.n; f0 += 16) {
         float2 v[16];
 #pragma unroll
         for (int f = 0; f < 16; ++f) v[f] = f0 + f < e.n ? __ldcs(src + (int64_t)(f0 + f) * pitch) : mu;
-        float2 sum[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};   // of eight frames each
 #pragma unroll
         for (int f = 0; f < 16; ++f)
             if (f0 + f < e.n) {
                 const float2 y = make_float2(v[f].x - mu.x, v[f].y - mu.y);
-                sum[f / 8] = __fadd2_rn(sum[f / 8], y);
+                if (SPLIT || f < 8) {
+                    sum.x += y.x;
+                    sum.y += y.y;
+                } else {
+                    half.x += y.x;
+                    half.y += y.y;
+                }
                 if (CHECK) {
                     const float2 c = CHECK == 2 ? v[f] : y;
                     amax = fmaxf(amax, fmaxf(fabsf(c.x), fabsf(c.y)));
                 }
                 carry[(int64_t)(f0 + f) * e.M_pad] = y;
             }
-        add_partial(tot, rest, sum[0]);
-        add_partial(tot, rest, sum[1]);
+        if (!SPLIT || (f0 & 16)) {
+            add_residual(&e.sum_res[m], sum);
+            sum = make_float2(0.f, 0.f);
+        }
+        if (!SPLIT && f0 + 8 < e.n) {
+            add_residual(&e.sum_res[m], half);
+            half = make_float2(0.f, 0.f);
+        }
     }
-    add_residual(&e.sum_res[m], tot, rest);
+    if (SPLIT) add_residual(&e.sum_res[m], sum);
     if (CHECK && amax * e.f16_scale > 65504.f) atomicOr(e.err, DEVERR_FP16_RANGE);
 }
 
 template <int B, int R, bool SPLIT, int CHECK>
 static cudaError_t launch_project_kernel(const ProjGroup &pg, cudaStream_t st) {
     using SM = ProjSmem<B, R, SPLIT>;
-    auto *kern = project_group_kernel<B, R, SPLIT, CHECK, false>;
-    if constexpr (CHECK != 2)   // (rare: one kernel for any number of entries)
-        if (pg.n == 1) kern = project_group_kernel<B, R, SPLIT, CHECK, true>;
+    auto *kern = pg.n == 1 ? project_group_kernel<B, R, SPLIT, CHECK, true> : project_group_kernel<B, R, SPLIT, CHECK, false>;
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -535,12 +561,11 @@ cudaError_t launch_project_group(ProjGroup &pg, int B, int R, bool split, cudaSt
     bool blocks = false;
     for (int i = 0; i < pg.n; ++i) blocks = blocks || pg.e[i].nblk > 0;
     if (!blocks) {
-        if (pg.check == 2)
-            carry_group_kernel<2><<<(unsigned)pg.groups, 128, 0, st>>>(pg);
-        else if (pg.check == 1)
-            carry_group_kernel<1><<<(unsigned)pg.groups, 128, 0, st>>>(pg);
-        else
-            carry_group_kernel<0><<<(unsigned)pg.groups, 128, 0, st>>>(pg);
+        void (*kern)(ProjGroup) = !split            ? carry_group_kernel<0, false>
+                                  : pg.check == 2   ? carry_group_kernel<2, true>
+                                  : pg.check == 1   ? carry_group_kernel<1, true>
+                                                    : carry_group_kernel<0, true>;
+        kern<<<(unsigned)pg.groups, 128, 0, st>>>(pg);
         return cudaGetLastError();
     }
 #define TACAW_PROJ(b, r) \

@@ -210,8 +210,10 @@ __device__ __forceinline__ void convert_tiled_rows(const FrameGeom &g, int n, in
     for (int t0 = 0; t0 < n;) {
         const int f0 = (s0 + t0) % bf;                 // first frame of the piece inside its block
         const int lead = ALIGNED ? 0 : f0 & 3;         // words of its first chunk before it
-        const int len = ALIGNED ? min(bf - f0, n - t0) : min(min(bf - f0, n - t0), PF - lead);
-        const int c0 = f0 / 4, end = lead + len, nc = ALIGNED ? len / 4 : (end + 3) / 4;
+        // (kShort: forms of the same numbers that leave 64 registers there; the other kernels were 4 to 7 % slower by them)
+        constexpr bool kShort = ALIGNED && PF == 16 && F16;
+        const int len = kShort ? min(bf - f0, n - t0) : min(min(bf - f0, n - t0), PF - lead);
+        const int c0 = f0 / 4, end = lead + len, nc = kShort ? len / 4 : (end + 3) / 4;
         float2 v[PF];                                  // by word of the piece's chunks; others stay at the mean
 #pragma unroll
         for (int i = 0; i < PF; ++i)
