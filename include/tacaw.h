@@ -87,8 +87,11 @@ typedef enum {
  * where the energies cover less than half of the band 1/dt, pushes may stage blocks of 32, 64 or 128
  * frames as their fewer coefficients on an orthonormal basis of that band (reconstruction error
  * 1e-7), which the contraction sums like frames.  The first push into a staging ring picks the form by
- * its length.  On both split paths the coefficients are fp16 hi + lo pieces under a power-of-two scale
- * per row, whatever the pieces of staged frames are; no input is refused for it.
+ * its length, so results depend on how a segment is split into pushes, to rounding (with plain frames and
+ * the mean kept they do not).  On both split paths the coefficients are fp16 hi + lo pieces under a
+ * power-of-two scale per row, whatever the pieces of staged frames are; no input is refused for it.
+ * Streams with such forms that keep their mean (subtract_mean 0) have the provisional mean taken out of
+ * their frames and added back in the spectra.
  * Twiddle phases are always reduced in FP64; the exact mean correction is FP64-derived. */
 typedef enum { TACAW_PREC_FP32 = 0, TACAW_PREC_SPLIT_BF16 = 1, TACAW_PREC_SPLIT_FP16 = 2 } tacaw_precision;
 
@@ -343,7 +346,9 @@ tacaw_status tacaw_set_adjoint_precision(tacaw_plan_t plan, int precision);
  * it is deferred, and the next segment's tacaw_finalize_async launches it together with the
  * conversion of that next segment's pushes, which two extra warps of the same launch do while
  * its tensor cores run (the pushes of a segment that follows a deferred one only record their
- * frame addresses; the frames must stay valid until that launch has run).  Each segment stages
+ * frame addresses; the frames must stay valid until that launch has run).  A segment whose first
+ * push picks a band-limited form is converted at push time instead, and the deferred contraction
+ * goes out at its finalize all the same.  Group pushes go as single ones.  Each segment stages
  * into one of two staging areas in turn: enabling allocates the second (TACAW_ERR_OOM if it
  * does not fit).  tacaw_drain launches a deferred contraction on its own; tacaw_finalize (the
  * waiting form) does so before it waits.  Results of a segment are complete once its deferred
@@ -354,7 +359,8 @@ tacaw_status tacaw_set_adjoint_precision(tacaw_plan_t plan, int precision);
 tacaw_status tacaw_set_pipelined_segments(tacaw_plan_t plan, int enable);
 
 /* Launches a deferred contraction (pipelined segments), on `stream`; no-op without one.
- * STATE while the current segment's pushes wait for it (finalize that segment first).       */
+ * STATE while the current segment has pushes (finalize that segment first: they may wait for the
+ * contraction).                                                                             */
 tacaw_status tacaw_drain(tacaw_plan_t plan, void *stream);
 
 /* Starts a new segment on every stream (e.g. the next probe batch or trajectory chunk):

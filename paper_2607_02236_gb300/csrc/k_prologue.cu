@@ -103,12 +103,12 @@ __host__ __device__ __forceinline__ int swz_word(int w, int64_t m, int bf, int s
     return ((((w >> 2) ^ sw)) << 2) | (w & 3);
 }
 
-// Blocks of 8 frames.  Staged frame slot s (s0 + t) goes to block s/bf, elements 2(s%bf), 2(s%bf)+1 of row m
-// (rows of 2*bf bf16 = 4*bf bytes; bf is 8, 16 or 32).
+// Staging blocks of 8 frames (longer ones: convert_tiled_rows).  Staged frame slot s (s0 + t) goes to block s/8,
+// elements 2(s%8), 2(s%8)+1 of row m (rows of 16 elements of 16 bits, 32 bytes).
 template <bool F16>
-__global__ void convert_split_kernel(FrameGeom g, int n, int s0, int bf, int64_t M_pad, const float2 *mu_hat,
-                                     double2 *sum_res, __nv_bfloat16 *A_hi, __nv_bfloat16 *A_lo, int swz,
-                                     float sc, uint32_t *err) {
+__global__ void convert_split_kernel(FrameGeom g, int n, int s0, int64_t M_pad, const float2 *mu_hat, double2 *sum_res,
+                                     __nv_bfloat16 *A_hi, __nv_bfloat16 *A_lo, int swz, float sc, uint32_t *err) {
+    constexpr int bf = 8;
     int64_t m = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (m >= g.M) return;
     const float2 *src = row_src(g, m);
@@ -118,7 +118,7 @@ __global__ void convert_split_kernel(FrameGeom g, int n, int s0, int bf, int64_t
     double sr = 0.0, si = 0.0;
     float amax = 0.f;
     int t = 0;
-    // leading frames up to the next block boundary
+    // leading frames up to the next block
     while (t < n && ((s0 + t) & 7)) {
         const int s = s0 + t;
         float2 v = __ldcs(src + (int64_t)t * g.pitch_frame);
@@ -132,7 +132,7 @@ __global__ void convert_split_kernel(FrameGeom g, int n, int s0, int bf, int64_t
         Lo[o] = l;
         ++t;
     }
-    // groups of 8 frames -> 32 bytes of the row of hi and of lo
+    // whole blocks -> 32 bytes of hi and of lo
     for (; t + 8 <= n; t += 8) {
         float2 v[8];
 #pragma unroll
@@ -430,8 +430,8 @@ static cudaError_t convert_split(const FrameGeom &g, int n, int s0, int bf, int6
         kern<<<grid, 128, 0, st>>>(g, n, s0, M_pad, mu_hat, sum_res, A_hi, A_lo, swz, sc, err);
         return cudaGetLastError();
     }
-    convert_split_kernel<F16><<<blocks_for(g.M, 256), 256, 0, st>>>(g, n, s0, bf, M_pad, mu_hat, sum_res, A_hi,
-                                                                    A_lo, swz, sc, err);
+    convert_split_kernel<F16><<<blocks_for(g.M, 256), 256, 0, st>>>(g, n, s0, M_pad, mu_hat, sum_res, A_hi, A_lo, swz,
+                                                                    sc, err);
     return cudaGetLastError();
 }
 

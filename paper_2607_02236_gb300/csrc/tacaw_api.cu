@@ -1727,7 +1727,7 @@ tacaw_status tacaw_drain(tacaw_plan_t p, void *stream) {
     tacaw_status c = check_plan(p);
     if (c != TACAW_OK) return c;
     if (p->deferred_pushes)
-        return fail(TACAW_ERR_STATE, "the segment's pushes wait for the pending contraction: finalize the segment first");
+        return fail(TACAW_ERR_STATE, "a segment follows the deferred contraction and has pushes: finalize the segment first");
     if (!p->pend.active) return TACAW_OK;
     return launch_pending(p, nullptr, static_cast<cudaStream_t>(stream));
 }
