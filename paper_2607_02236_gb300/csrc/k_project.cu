@@ -60,7 +60,7 @@ __device__ __forceinline__ void proj_copy(float2 *dst, const float2 *src, int by
 // With frames of size a and unit rounding u: on the FP32 path sums of 16 frames from four sums of four (68 a u, two sums
 // of eight one by one 70) are added this way; FP64 adds would be two additions and two conversions each, on a pipe with
 // a 64th of the FP32 rate.  On the split path a block's sums of four frames are added in FP32: 668 a u for 64 frames,
-// two sums of 32 one by one 1054.  Cost: the FP32 scan (blocks of 128 frames, R 36) 6.16 ms instead of 6.05.
+// two sums of 32 one by one 1054.  Cost: the FP32 scan (blocks of 128 frames, R 36) 6.14 ms instead of 6.08.
 __device__ __forceinline__ void add_partial(float2 &tot, float2 &rest, float2 part) {
     const float2 t = __fadd2_rn(tot, part);
     const float2 b = __fadd2_rn(t, make_float2(-tot.x, -tot.y));       // the part as it went in
@@ -463,9 +463,9 @@ __global__ void __launch_bounds__(128, ProjSmem<B, R, SPLIT>::kCtas)
 }
 
 // Pushes that complete no block: their frames' residuals go to the carry, 8 bytes read and 8 written a
-// (row, frame) at full occupancy; their sums to FP64 every 32 frames (SPLIT) or 8, straight to memory: kept in
+// (row, frame) at full occupancy; their sums to FP64 every 32 frames (SPLIT) or 16 (by fours), straight to memory: kept in
 // registers over the push (add_partial) the longer code cost more than the atomics (16-frame pushes of 10^4 rows
-// x 2048 frames, FP32: 1.47 ms a segment against 1.30).  CTA b: rows 128 (b - group_begin) .. of its entry.
+// x 2048 frames, FP32: 1.47 ms a segment against 1.29).  CTA b: rows 128 (b - group_begin) .. of its entry.
 template <int CHECK, bool SPLIT>
 __global__ void __launch_bounds__(128, 8) carry_group_kernel(const __grid_constant__ ProjGroup pg) {
     int i = 0;
@@ -477,36 +477,29 @@ __global__ void __launch_bounds__(128, 8) carry_group_kernel(const __grid_consta
     const float2 *src = e.g.base + proj_row(e.g, m);
     float2 *carry = e.carry + m + (int64_t)e.c0 * e.M_pad;
     const float2 mu = e.mu_hat[m];
-    float2 sum = make_float2(0.f, 0.f), half = sum;
+    float2 sum = make_float2(0.f, 0.f);
     float amax = 0.f;
     for (int f0 = 0; f0 < e.n; f0 += 16) {
-        float2 v[16];
+        float2 v[16], four[4] = {};
 #pragma unroll
         for (int f = 0; f < 16; ++f) v[f] = f0 + f < e.n ? __ldcs(src + (int64_t)(f0 + f) * pitch) : mu;
 #pragma unroll
         for (int f = 0; f < 16; ++f)
             if (f0 + f < e.n) {
                 const float2 y = make_float2(v[f].x - mu.x, v[f].y - mu.y);
-                if (SPLIT || f < 8) {
-                    sum.x += y.x;
-                    sum.y += y.y;
-                } else {
-                    half.x += y.x;
-                    half.y += y.y;
-                }
+                float2 &s = SPLIT ? sum : four[f / 4];
+                s.x += y.x;
+                s.y += y.y;
                 if (CHECK) {
                     const float2 c = CHECK == 2 ? v[f] : y;
                     amax = fmaxf(amax, fmaxf(fabsf(c.x), fabsf(c.y)));
                 }
                 carry[(int64_t)(f0 + f) * e.M_pad] = y;
             }
+        if (!SPLIT) sum = __fadd2_rn(__fadd2_rn(four[0], four[1]), __fadd2_rn(four[2], four[3]));
         if (!SPLIT || (f0 & 16)) {
             add_residual(&e.sum_res[m], sum);
             sum = make_float2(0.f, 0.f);
-        }
-        if (!SPLIT && f0 + 8 < e.n) {
-            add_residual(&e.sum_res[m], half);
-            half = make_float2(0.f, 0.f);
         }
     }
     if (SPLIT) add_residual(&e.sum_res[m], sum);
