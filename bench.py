@@ -237,7 +237,8 @@ def step_roofline(bytes_step, ms_step, kernel_ms, kname, launches_per_step):
     hbm = peaks.get("hbm_gbs")
     ach = bytes_step / (ms_step * 1e-3) / 1e9
     return {"bound": "hbm", "achieved": ach, "peak": hbm, "unit": "GB/s", "frac": ach / hbm if hbm else None,
-            "traffic": None, "kernel": kname, "kernel_ms": kernel_ms, "launches_per_step": launches_per_step,
+            "traffic": None, "kernel": "whole step: pushes, contraction (" + kname + "), spectra",
+            "kernel_ms": kernel_ms, "kernel_ms_of": kname, "launches_per_step": launches_per_step,
             "bytes_per_step": bytes_step, "ms_per_step": ms_step,
             "peak_source": f"{src} copy bandwidth (MEASURED_PEAKS.json hbm_gbs)"}
 
