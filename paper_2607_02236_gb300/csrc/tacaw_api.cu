@@ -1155,6 +1155,8 @@ tacaw_status finish_segment(tacaw_plan_s *p, UserStream &u, Stream &s, cudaStrea
     tacaw_status r = run_flush(p, s, FLUSH_FINAL, u.I_acc, nullptr, st);
     if (r != TACAW_OK) return r;
     CU_CHECK(p, cudaMemsetAsync(s.sum_res, 0, sizeof(double2) * s.M, st), "reset sums");
+    // the lane's next segment may be one that keeps its mean in plain frames (split FP16)
+    if (p->f16 && s.shifted) CU_CHECK(p, cudaMemsetAsync(s.mu_hat, 0, sizeof(float2) * s.M, st), "reset mean");
     s.pushed = s.staged = s.stage_start = s.flushes = 0;
     s.form = -1;
     s.seg += u.lanes;

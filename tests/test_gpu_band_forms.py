@@ -556,3 +556,23 @@ def test_captured_segment_in_blocks(precision):
             torch.cuda.synchronize()
             assert np.array_equal(I.cpu().numpy(), want[k])
     assert_exact(want[1].reshape(-1, ROWS), frs[1], cfg)
+
+
+def test_split_fp16_welch_segments_of_both_kinds():
+    """A lane's first segment in blocks, its kept mean taken out, the next one as plain frames of the other sign at
+    0.92 of the fp16 range: nothing of the first one's mean is left in the second's conversion."""
+    from paper_2607_02236_gb300 import TacawPlan
+    cfg = config(512, 1000, 150.0, subtract_mean=False, welch_segments=2, welch_stride=512)
+    fr = waves(1024, 27, elastic=0.0)
+    fr[:512] += 14.7
+    fr[512:] -= 14.7
+    with TacawPlan([cfg], precision="split_fp16") as plan:
+        push_all(plan, fr, [64], 0, 64)
+        assert ring_form(plan) == 64
+        push_all(plan, fr, [64], 64, 512)
+        push_all(plan, fr, [8], 512, 520)
+        assert ring_form(plan) == 0
+        push_all(plan, fr, [8], 520)
+        I, _ = finish(plan)
+    ref = oracle.welch_forward(fr[:, PIX].cpu().numpy()[None, :, None, :], 512, 512, E_meV=cfg.E_meV, subtract_mean=False)
+    assert rel_err_peak(I[:, PIX], ref.I[0, :, 0]) <= TOL
